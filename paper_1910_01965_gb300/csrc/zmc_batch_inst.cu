@@ -14,6 +14,9 @@
 // single-scan kernel; the order of the compensated additions does not depend
 // on the blocking in any case, so results stay bit-identical to solo runs.
 #include "zmc_scan_kernel.cuh"
+#if ZMC_INST_PREC == 0
+#include "zmc_integrands_fixed.cuh"
+#endif
 
 #ifndef ZMC_INST_PREC
 #error "ZMC_INST_PREC must be defined"
@@ -38,7 +41,8 @@ namespace zmc {
 // allocation instead of the union of all 48 bodies (one call per tile).
 template <int N, class F, int PREC>
 __device__ __noinline__ void batch_tile(const ScanArgs& a, const BatchTile& t, bool restage,
-                                           double* smem, float* dimc, double* red) {
+                                           double* smem, float* dimc, const int64_t* fxc,
+                                           const int64_t* fxe, double* red) {
   // Lists / tables of this scan (kept when the previous tile was the same scan).
   const void* table = nullptr;
   if (restage) {
@@ -56,9 +60,11 @@ __device__ __noinline__ void batch_tile(const ScanArgs& a, const BatchTile& t, b
   const int local = threadIdx.x >> a.lanes_log2;
   const bool active = local < t.units;
   const int64_t us = t.first_us + local;
-  LaneAcc<PREC> acc;
-  if (active) unit_split_lane<N, F, PREC>(a, rk0, rk1, table, dimc, us, lane, acc);
-  double s1 = acc.sum1(), s2 = acc.sum2();
+  double s1 = 0.0, s2 = 0.0;
+  if (active)
+    unit_split_lane<N, F, PREC>(a, rk0, rk1, table, dimc,
+                                FxOf<F, PREC>::kTable == kFxExpTable ? fxe : fxc, us, lane, s1,
+                                s2);
   reduce_unit_split(a, s1, s2, red);
   if (lane == 0 && active && ZMC_CHECK(a.dbg, us >= 0 && us < a.n_us, kDbgPartialSlot, us)) {
     a.partial[2 * us] = s1;
@@ -68,7 +74,7 @@ __device__ __noinline__ void batch_tile(const ScanArgs& a, const BatchTile& t, b
 
 #define ZMC_CASE_N(gid, F, n)                                                        \
   case (gid)*8 + (n)-1:                                                              \
-    batch_tile<n, F<n>, ZMC_INST_PREC>(a, t, restage, smem, dimc, red);              \
+    batch_tile<n, F<n>, ZMC_INST_PREC>(a, t, restage, smem, dimc, fxc, fxe, red);              \
     break;
 #define ZMC_CASES(gid, F)                                                            \
   ZMC_CASE_N(gid, F, 1) ZMC_CASE_N(gid, F, 2) ZMC_CASE_N(gid, F, 3)                  \
@@ -82,6 +88,13 @@ batch_kernel(const __grid_constant__ BatchArgs b) {
   __shared__ double red[64];
   __shared__ float dimc[3 * ZMC_MAX_N];
   __shared__ long long s_tile;
+  const int64_t *fxc = nullptr, *fxe = nullptr;
+#if ZMC_INST_PREC == 0
+  __shared__ int64_t fx_tables[kFxCosEntries + kFxExpEntries];
+  fx_fill_tables(fx_tables);  // the first barrier of the loop is behind it
+  fxc = fx_tables;
+  fxe = fx_tables + kFxCosEntries;
+#endif
   int staged = -1;  // scan whose lists/tables are in shared memory
   for (;;) {
     if (threadIdx.x == 0) s_tile = static_cast<long long>(atomicAdd(b.counter, 1ull));
@@ -113,13 +126,31 @@ batch_kernel(const __grid_constant__ BatchArgs b) {
 #define ZMC_BATCH_OCC2(p) batch_occupancy_p##p
 #define ZMC_BATCH_OCC(p) ZMC_BATCH_OCC2(p)
 
+// Shared memory above the default 48 KB has to be asked for; the FP64 kernel
+// holds both fixed-point tables beside the scans' lists.
+static cudaError_t allow_smem(size_t smem) {
+#if ZMC_INST_PREC == 0
+  const size_t fixed = (kFxCosEntries + kFxExpEntries) * sizeof(int64_t) + 1024;
+#else
+  const size_t fixed = 1024;
+#endif
+  if (smem + fixed <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(batch_kernel<ZMC_INST_PREC>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(smem));
+}
+
 int ZMC_BATCH_FN(ZMC_INST_PREC)(const BatchArgs& b, int grid, int block, size_t smem,
                                 void* stream) {
+  const cudaError_t e = allow_smem(smem);
+  if (e != cudaSuccess) return static_cast<int>(e);
   batch_kernel<ZMC_INST_PREC><<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(b);
   return static_cast<int>(cudaGetLastError());
 }
 
 int ZMC_BATCH_OCC(ZMC_INST_PREC)(int block, size_t smem, int* out) {
+  const cudaError_t e = allow_smem(smem);
+  if (e != cudaSuccess) return static_cast<int>(e);
   return static_cast<int>(
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, batch_kernel<ZMC_INST_PREC>, block,
                                                     smem));

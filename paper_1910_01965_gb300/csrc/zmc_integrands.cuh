@@ -67,6 +67,11 @@ __device__ __forceinline__ double field_unit<double>(uint32_t v) {
   return __longlong_as_double(
       static_cast<long long>(0x3FF0000000000000ull | (static_cast<uint64_t>(v) << 29)));
 }
+// The fixed-point functors take the field itself.
+template <>
+__device__ __forceinline__ uint32_t field_unit<uint32_t>(uint32_t v) {
+  return v;
+}
 
 __device__ __forceinline__ float ex2_approx(float v) {
   float out;
@@ -75,6 +80,10 @@ __device__ __forceinline__ float ex2_approx(float v) {
 }
 
 // ------------------------------------------------------------------ FP64 --
+// The functors with the suffix Wide take any parameters and box; the FP64
+// kernels evaluate the same integrands in fixed point where those are in range
+// (zmc_integrands_fixed.cuh) and use these elsewhere.
+//
 // FP64 functors fold the affine steps in y into per-unit constants the same way
 // the FP32 ones do: y = (b - a) f + A with A = a - (b - a)(1 - 2^-24), so each
 // dimension costs one DFMA before the integrand's own arithmetic.  The result
@@ -96,7 +105,7 @@ struct Const64 {
 
 // cos(x y) = cos(B f + C), B = x (b - a), C = x A.
 template <int N>
-struct CosProd64 {
+struct CosProd64Wide {
   static constexpr bool kPerDim = true;
   static constexpr bool kTable = false;
   static constexpr bool kUsesSamples = true;
@@ -119,7 +128,7 @@ struct CosProd64 {
 
 // y - x = W f + C, C = A - x.
 template <int N>
-struct Gauss64 {
+struct Gauss64Wide {
   static constexpr bool kPerDim = true;
   static constexpr bool kTable = false;
   static constexpr bool kUsesSamples = true;
@@ -172,7 +181,7 @@ struct Poly64 {
 };
 
 template <int N>
-struct Osc64 {
+struct Osc64Wide {
   static constexpr bool kPerDim = true;
   static constexpr bool kTable = false;
   static constexpr bool kUsesSamples = true;
@@ -200,7 +209,7 @@ struct Osc64 {
 
 // sin(sum_k W_k f_k + C0), C0 = sum_k A_k + sum_l x_l.
 template <int N>
-struct SinSum64 {
+struct SinSum64Wide {
   static constexpr bool kPerDim = false;
   static constexpr bool kTable = false;
   static constexpr bool kUsesSamples = true;

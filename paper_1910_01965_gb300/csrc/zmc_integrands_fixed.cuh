@@ -1,0 +1,266 @@
+// zmc_integrands_fixed.cuh — the FP64 integrands in 64-bit fixed point.
+//
+// Each functor evaluates its integrand from the sample's 23-bit fields with the
+// arithmetic of zmc_fixed64.cuh.  `set`/`finish` turn the box and the
+// parameters into fixed-point constants and decide (`ok`) whether they are in
+// range; out of range, and for NaN or infinite parameters, the unit is sampled
+// by the FP64 functor named in FxOf (zmc_integrands.cuh, suffix Wide).
+//
+// With u = (2 v + 1) 2^-24 and w = b - a (rounded to FP64, as there):
+// y = a + w 2^-24 + (w 2^-23) v.
+#pragma once
+
+#include "zmc_fixed64.cuh"
+#include "zmc_scan_kernel.cuh"
+
+namespace zmc {
+
+// Lane sums of values g with |g| <= 1, held as 2^62 g + 2^31: exact sums of g
+// and of g^2 to 2^-60 (rounded), converted to FP64 once per lane.  Integer sums
+// cost 5 adds against 64 SMSP clocks for one FP64 add.
+struct FxLaneAcc {
+  FxSum a1, a2;
+  uint64_t n = 0;
+  __device__ __forceinline__ void sum(int64_t g) {
+    a1.add(g);
+    const int32_t h = fx_top(g);
+    const int32_t t = fx_mulhi(h, fx_low(g));
+    a2.add(fx_wide(h, h) + (2 * t + 1));
+  }
+  __device__ __forceinline__ void add(int64_t g) {
+    sum(g);
+    n += 1;
+  }
+  __device__ __forceinline__ void add2(int64_t a, int64_t b) {
+    sum(a);
+    sum(b);
+    n += 2;
+  }
+  template <int K>
+  __device__ __forceinline__ void add_group(const int64_t* v) {
+#pragma unroll
+    for (int i = 0; i < K; ++i) sum(v[i]);
+    n += K;
+  }
+  __device__ __forceinline__ double sum1() const { return a1.value(n, 62); }
+  __device__ __forceinline__ double sum2() const { return a2.value(0, 60); }
+};
+
+// prod_k cos(x_k y_k): a 96-bit phase per dimension.  In range: phases below
+// 2^20 radians.
+template <int N>
+struct CosProd64 {
+  static constexpr bool kPerDim = true;
+  static constexpr bool kTable = false;
+  static constexpr bool kUsesSamples = true;
+  static constexpr int kCallsInFlight = 1;
+  static constexpr int kFixedM = 0;
+  using unit_t = uint32_t;
+  const int64_t* fx;
+  bool ok = true;
+  uint32_t b0[N], b1[N], b2[N];
+  uint64_t c[N];
+  __device__ void set(int i, double xi, double ai, double bi) {
+    const double w = bi - ai;
+    ok = ok && fx_below(xi * w, 20) && fx_below(xi * ai, 20);
+    const FxTurns b = fx_turns_mul(xi, w, -23);
+    b0[i] = b.w0;
+    b1[i] = b.w1;
+    b2[i] = b.w2;
+    c[i] = fx_phase0(fx_turns_add(fx_turns_mul(xi, ai, 0), fx_turns_sar(b, 1)));
+  }
+  __device__ int64_t eval(const uint32_t* v) const {
+    int64_t g = fx_cos(fx_phase_step(c[0], v[0], b0[0], b1[0], b2[0]), fx);
+#pragma unroll
+    for (int k = 1; k < N; ++k)
+      g = fx_mul62(g, fx_cos(fx_phase_step(c[k], v[k], b0[k], b1[k], b2[k]), fx));
+    return g;
+  }
+};
+
+// sin(sum_k y_k + sum_l x_l) as the cosine a quarter turn behind.  In range:
+// the parameters' sum and the box's sides and corner below 2^20.
+template <int N>
+struct SinSum64 {
+  static constexpr bool kPerDim = false;
+  static constexpr bool kTable = false;
+  static constexpr bool kUsesSamples = true;
+  static constexpr int kCallsInFlight = 1;
+  static constexpr int kFixedM = 0;
+  using unit_t = uint32_t;
+  const int64_t* fx;
+  bool ok = true;
+  double xsum;
+  uint32_t b0[N], b1[N], b2[N];
+  uint64_t c;
+  __device__ void add(double xi) { xsum += xi; }
+  __device__ void finish(const double* lo, const double* hi) {
+    ok = fx_below(xsum, 20);
+    FxTurns t = fx_turns_add(fx_turns(xsum, 0), {0, 0, 0xC0000000u});
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const double w = hi[k] - lo[k];
+      ok = ok && fx_below(lo[k], 20) && fx_below(w, 20);
+      const FxTurns b = fx_turns(w, -23);
+      b0[k] = b.w0;
+      b1[k] = b.w1;
+      b2[k] = b.w2;
+      t = fx_turns_add(t, fx_turns_add(fx_turns(lo[k], 0), fx_turns_sar(b, 1)));
+    }
+    c = fx_phase0(t);
+  }
+  __device__ int64_t eval(const uint32_t* v) const {
+    uint64_t th = c;
+#pragma unroll
+    for (int k = 0; k < N; ++k) th = fx_phase_step(th, v[k], b0[k], b1[k], b2[k]);
+    return fx_cos(th, fx);
+  }
+};
+
+// frac(0.1 a b 2^k / (2 pi)) from the exact products.
+__device__ __forceinline__ FxTurns fx_turns_quad(double a, double b, int k) {
+  const double p = a * b;
+  return fx_turns_add(fx_turns_mul(kOscQuad, p, k), fx_turns_mul(kOscQuad, fma(a, b, -p), k));
+}
+
+// cos(sum_k x_k y_k + 0.1 y_k^2).  In turns, dimension k adds
+//   (q v + l) v + const,  q = 0.1 w^2 2^-46,  l = (x w + 0.2 a w) 2^-23 + q,
+// by Horner's rule with q 2^23 and l held to 96 bits.  In range: box within
+// 2^10 of the origin, x w and x a below 2^20.
+template <int N>
+struct Osc64 {
+  static constexpr bool kPerDim = true;
+  static constexpr bool kTable = false;
+  static constexpr bool kUsesSamples = true;
+  static constexpr int kCallsInFlight = 1;
+  static constexpr int kFixedM = 0;
+  using unit_t = uint32_t;
+  const int64_t* fx;
+  bool ok = true;
+  uint32_t q0[N], q1[N], q2[N];  // q 2^23, below 1/2
+  uint32_t l0[N], l1[N], l2[N];
+  uint64_t c = uint64_t(1) << 52;  // half a table step
+  __device__ void set(int i, double xi, double ai, double bi) {
+    const double w = bi - ai;
+    ok = ok && fx_below(xi * w, 20) && fx_below(xi * ai, 20) && fx_below(ai, 10) &&
+         fx_below(w, 10);
+    const FxTurns xw = fx_turns_mul(xi, w, -23);
+    const FxTurns q = fx_turns_quad(w, w, -23);
+    const FxTurns aw = fx_turns_quad(ai, w, -22);
+    const FxTurns lin = fx_turns_add(xw, aw);
+    const FxTurns l = fx_turns_add(lin, fx_turns_sar(q, 23));
+    q0[i] = q.w0;
+    q1[i] = q.w1;
+    q2[i] = q.w2;
+    l0[i] = l.w0;
+    l1[i] = l.w1;
+    l2[i] = l.w2;
+    // x a + 0.1 a^2 + half a field of the linear part + 0.1 w^2 2^-48
+    const FxTurns k0 = fx_turns_add(fx_turns_mul(xi, ai, 0), fx_turns_quad(ai, ai, 0));
+    const FxTurns k1 = fx_turns_add(fx_turns_sar(lin, 1), fx_turns_sar(q, 25));
+    const FxTurns k = fx_turns_add(k0, k1);
+    c += (static_cast<uint64_t>(k.w2) << 32) | k.w1;
+  }
+  __device__ int64_t eval(const uint32_t* v) const {
+    uint64_t th = c;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const uint32_t f = v[k] << 9;  // v 2^-23 as a 32-bit fraction
+      const uint64_t p1 = fx_uwide(f, q1[k]) + fx_umulhi(f, q0[k]);
+      const uint64_t p2 = fx_uwide(f, q2[k]) + (p1 >> 32);
+      const FxTurns s = fx_turns_add({static_cast<uint32_t>(p1), static_cast<uint32_t>(p2),
+                                      static_cast<uint32_t>(p2 >> 32)},
+                                     {l0[k], l1[k], l2[k]});
+      th = fx_phase_step(th, v[k], s.w0, s.w1, s.w2);
+    }
+    return fx_cos(th, fx);
+  }
+};
+
+// 2^-q, q = sum_k d_k^2, d = scale (y - x) as a signed 5.59-bit number.  In
+// range: |d| < 15.9 over the box in every dimension and q < 990, so that 2^-q
+// is a normal double.  The sums stay FP64 (the FP64 unit is otherwise idle).
+template <int N>
+struct Gauss64 {
+  static constexpr bool kPerDim = true;
+  static constexpr bool kTable = false;
+  static constexpr bool kUsesSamples = true;
+  static constexpr int kCallsInFlight = 1;
+  static constexpr int kFixedM = 0;
+  using unit_t = uint32_t;
+  // 2^61 sqrt(log2(e) / 0.18)
+  static constexpr uint64_t kScale61 = 0x5a9825b501cd145cull;
+  const int64_t* fx;
+  bool ok = true;
+  float qmax = 0.0f;
+  uint32_t w0[N], w1[N];
+  int64_t c[N];
+  __device__ void set(int i, double xi, double ai, double bi) {
+    const double w = bi - ai;
+    // a - x as an exact sum of two doubles
+    const double s = ai - xi, bb = s - ai;
+    const double e = (ai - (s - bb)) + (-xi - bb);
+    const float m = 2.8310728f * fmaxf(fabsf(static_cast<float>(s)),
+                                       fabsf(static_cast<float>(bi - xi)));
+    qmax = fmaf(m, m, qmax);
+    ok = ok && m < 15.9f && qmax < 990.0f && xi == xi;  // fmaxf drops a NaN
+    const uint64_t cw = static_cast<uint64_t>(fx_scale59(w, kScale61));
+    w0[i] = static_cast<uint32_t>(cw);
+    w1[i] = static_cast<uint32_t>(cw >> 32);
+    c[i] = fx_scale59(s, kScale61) + fx_scale59(e, kScale61) +
+           static_cast<int64_t>(((cw >> 23) + 1) >> 1) + kFxBias;
+  }
+  __device__ double eval(const uint32_t* v) const {
+    uint64_t q = uint64_t(1) << 42;  // half a table step
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const uint32_t f = v[k] << 9;  // v 2^-23 as a 32-bit fraction
+      const int64_t d = c[k] + static_cast<int64_t>(fx_uwide(f, w1[k]) + fx_umulhi(f, w0[k]));
+      const int32_t h = fx_top(d);
+      const int32_t t = fx_mulhi(h, fx_low(d));
+      q += static_cast<uint64_t>(fx_wide(h, h) + (2 * t + 1));
+    }
+    return fx_exp2neg(q, fx);
+  }
+};
+
+__device__ __forceinline__ void fx_fill(int64_t* dst, const int64_t* src, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
+}
+
+// Both tables, the cosines first (the batched kernel).
+__device__ __forceinline__ void fx_fill_tables(int64_t* dst) {
+  fx_fill(dst, kFxTables.c, kFxCosEntries);
+  fx_fill(dst + kFxCosEntries, kFxTables.e, kFxExpEntries);
+}
+
+template <class W>
+struct FxCosOf {
+  static constexpr int kTable = kFxCosTable;
+  static constexpr int kEntries = kFxCosEntries;
+  static constexpr size_t kStaticBytes = kEntries * sizeof(int64_t);
+  using Wide = W;
+  using Acc = FxLaneAcc;
+  static __device__ __forceinline__ void fill(int64_t* dst) {
+    fx_fill(dst, kFxTables.c, kEntries);
+  }
+};
+template <int N>
+struct FxOf<CosProd64<N>, kPrecFP64> : FxCosOf<CosProd64Wide<N>> {};
+template <int N>
+struct FxOf<SinSum64<N>, kPrecFP64> : FxCosOf<SinSum64Wide<N>> {};
+template <int N>
+struct FxOf<Osc64<N>, kPrecFP64> : FxCosOf<Osc64Wide<N>> {};
+template <int N>
+struct FxOf<Gauss64<N>, kPrecFP64> {
+  static constexpr int kTable = kFxExpTable;
+  static constexpr int kEntries = kFxExpEntries;
+  static constexpr size_t kStaticBytes = kEntries * sizeof(int64_t);
+  using Wide = Gauss64Wide<N>;
+  using Acc = LaneAcc<kPrecFP64>;
+  static __device__ __forceinline__ void fill(int64_t* dst) {
+    fx_fill(dst, kFxTables.e, kEntries);
+  }
+};
+
+}  // namespace zmc

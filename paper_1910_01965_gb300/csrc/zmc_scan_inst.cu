@@ -2,6 +2,9 @@
 // one integrand, N = 1..8.  Compiled once per (ZMC_INST_PREC, ZMC_INST_GID)
 // pair so that the 144 kernels build in parallel.
 #include "zmc_scan_kernel.cuh"
+#if ZMC_INST_PREC == 0
+#include "zmc_integrands_fixed.cuh"
+#endif
 
 #ifndef ZMC_INST_PREC
 #error "ZMC_INST_PREC must be defined"

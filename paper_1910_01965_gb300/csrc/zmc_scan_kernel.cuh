@@ -35,6 +35,14 @@ enum { kPrecFP64 = ZMC_FP64, kPrecFP32 = ZMC_FP32, kPrecFP32K = ZMC_FP32_KAHAN }
 // ZMC_CALLS_IN_FLIGHT, when defined, overrides every functor's kCallsInFlight
 // (independent Philox calls per lane per loop block in the FP32 paths).
 
+// Fixed-point tables a functor reads from shared memory (0: none).
+enum { kFxNone = 0, kFxCosTable = 1, kFxExpTable = 2 };
+
+// The fixed-point functors specialise this: their table, their lane sums and
+// the FP64 functor that takes the parameters outside their range.
+template <class F, int PREC>
+struct FxOf;
+
 template <int PREC>
 struct LaneAcc;
 
@@ -133,6 +141,13 @@ struct LaneAcc<kPrecFP32K> {
   __device__ __forceinline__ double sum2() const {
     return static_cast<double>(s2) - static_cast<double>(c2);
   }
+};
+
+template <class F, int PREC>
+struct FxOf {
+  static constexpr int kTable = kFxNone;
+  static constexpr size_t kStaticBytes = 0;
+  using Acc = LaneAcc<PREC>;
 };
 
 // List that staged value `idx` belongs to.
@@ -269,12 +284,12 @@ __device__ __forceinline__ auto eval_sample(const F& f, const uint32_t* r, int g
 // G = 5, each group's five samples enter in one step (LaneAcc::add_group), in
 // group order; with G = 1, consecutive groups are paired and a last unpaired
 // group enters alone.
-template <int N, class F, int PREC>
+template <int N, class F, int PREC, class Acc>
 __device__ __forceinline__ void lane_groups(const uint32_t* __restrict__ rk0,
                                             const uint32_t* __restrict__ rk1,
                                             const PhiloxUnit& pu, const F& f, uint32_t q,
                                             uint32_t q_end, uint32_t step,
-                                            LaneAcc<PREC>& acc) {
+                                            Acc& acc) {
   constexpr int G = group_samples(N);
   constexpr int C = group_calls(N);
   // Groups per loop block: about kCallsInFlight independent Philox chains
@@ -308,7 +323,7 @@ __device__ __forceinline__ void lane_groups(const uint32_t* __restrict__ rk0,
   };
   if constexpr (G > 1) {
     constexpr int U = kBlock;
-    using T = typename F::unit_t;
+    using T = decltype(eval_sample<N>(f, static_cast<const uint32_t*>(nullptr), 0));
     auto consume = [&](const auto& r) {
       constexpr int V = sizeof(r) / sizeof(r[0]);
 #pragma unroll
@@ -383,11 +398,11 @@ __device__ __forceinline__ void lane_groups(const uint32_t* __restrict__ rk0,
 
 // The ragged last group of a unit when G does not divide S: its valid samples
 // enter one at a time.
-template <int N, class F, int PREC>
+template <int N, class F, class Acc>
 __device__ __forceinline__ void lane_tail_group(const uint32_t* __restrict__ rk0,
                                                 const uint32_t* __restrict__ rk1,
                                                 const PhiloxUnit& pu, const F& f, uint32_t q,
-                                                int valid, LaneAcc<PREC>& acc) {
+                                                int valid, Acc& acc) {
   constexpr int G = group_samples(N);
   constexpr int C = group_calls(N);
   uint32_t r[4 * C];
@@ -398,15 +413,60 @@ __device__ __forceinline__ void lane_tail_group(const uint32_t* __restrict__ rk0
     if (g < valid) acc.add(eval_sample<N>(f, r, g));
 }
 
+// Sums of one lane over its part of unit-split `split` of unit (p, t).
+template <int N, class F, int PREC, class Acc>
+__device__ __forceinline__ void sample_unit(const ScanArgs& a, const uint32_t* rk0,
+                                            const uint32_t* rk1, const F& f, int64_t p,
+                                            uint32_t t, int64_t split, int lane, Acc& acc) {
+  constexpr int G = group_samples(N);
+  const int64_t q0 = split * a.gps;
+  const int64_t q1 = min(q0 + a.gps, a.ngroups);
+  if constexpr (!F::kUsesSamples) {
+    // g does not depend on y: the stream is not drawn at all.
+    for (int64_t q = q0 + lane; q < q1; q += a.lanes) {
+      const int64_t left = a.S - q * G;
+      const int cnt = left < G ? static_cast<int>(left) : G;
+      for (int g = 0; g < cnt; ++g) acc.add(f.eval(nullptr));
+    }
+  } else {
+    const PhiloxUnit pu = philox_unit(rk0, rk1, static_cast<uint64_t>(p), t);
+    const int64_t nfull = a.S / G;
+    const int64_t qf = min(q1, nfull);
+    if (q0 + lane < qf)
+      lane_groups<N, F, PREC>(rk0, rk1, pu, f, static_cast<uint32_t>(q0 + lane),
+                              static_cast<uint32_t>(qf), static_cast<uint32_t>(a.lanes),
+                              acc);
+    if (G > 1) {
+      const int valid = static_cast<int>(a.S - nfull * G);
+      if (valid > 0 && nfull >= q0 && nfull < q1 && ((nfull - q0) & (a.lanes - 1)) == lane)
+        lane_tail_group<N, F>(rk0, rk1, pu, f, static_cast<uint32_t>(nfull), valid, acc);
+    }
+  }
+}
+
+// The same with an FP64 functor for parameters outside a fixed-point functor's
+// range.  Not inlined, so that it takes no registers from the usual path.
+template <int N, class F, int PREC>
+__device__ __noinline__ void sample_unit_wide(const ScanArgs& a, const void* table, int64_t p,
+                                              uint32_t t, int64_t split, int lane, double& s1,
+                                              double& s2) {
+  F f{};
+  load_params<N>(a, table, static_cast<const float*>(nullptr), p, f);
+  LaneAcc<PREC> acc;
+  sample_unit<N, F, PREC>(a, a.rk0, a.rk1, f, p, t, split, lane, acc);
+  s1 = acc.sum1();
+  s2 = acc.sum2();
+}
+
 // Work of one lane for unit-split `us`: decode, prepare, sample, sum.
 // rk0/rk1 are the ten Philox round keys (parameter space in the single-scan
-// kernel, registers in the batched one).
+// kernel, registers in the batched one); fx the fixed-point functors' table.
 template <int N, class F, int PREC>
 __device__ __forceinline__ void unit_split_lane(const ScanArgs& a, const uint32_t* rk0,
                                                 const uint32_t* rk1, const void* table,
-                                                const float* dimc, int64_t us, int lane,
-                                                LaneAcc<PREC>& acc) {
-  constexpr int G = group_samples(N);
+                                                const float* dimc, const int64_t* fx,
+                                                int64_t us, int lane, double& s1,
+                                                double& s2) {
   const int64_t unit = us / a.splits;
   const int64_t split = us - unit * a.splits;
   const int64_t lp = unit / a.T;
@@ -417,31 +477,18 @@ __device__ __forceinline__ void unit_split_lane(const ScanArgs& a, const uint32_
 
   F f{};
   load_params<N>(a, table, dimc, p, f);
-  if constexpr (!F::kUsesSamples) {
-    // g does not depend on y: the stream is not drawn at all.
-    const int64_t q0 = split * a.gps;
-    const int64_t q1 = min(q0 + a.gps, a.ngroups);
-    for (int64_t q = q0 + lane; q < q1; q += a.lanes) {
-      const int64_t left = a.S - q * G;
-      const int cnt = left < G ? static_cast<int>(left) : G;
-      for (int g = 0; g < cnt; ++g) acc.add(f.eval(nullptr));
+  if constexpr (FxOf<F, PREC>::kTable != kFxNone) {
+    if (!f.ok) {
+      sample_unit_wide<N, typename FxOf<F, PREC>::Wide, PREC>(a, table, p, t, split, lane, s1,
+                                                              s2);
+      return;
     }
-  } else {
-    const PhiloxUnit pu = philox_unit(rk0, rk1, static_cast<uint64_t>(p), t);
-    const int64_t q0 = split * a.gps;
-    const int64_t q1 = min(q0 + a.gps, a.ngroups);
-    const int64_t nfull = a.S / G;
-    const int64_t qf = min(q1, nfull);
-    if (q0 + lane < qf)
-      lane_groups<N, F, PREC>(rk0, rk1, pu, f, static_cast<uint32_t>(q0 + lane),
-                              static_cast<uint32_t>(qf), static_cast<uint32_t>(a.lanes),
-                              acc);
-    if (G > 1) {
-      const int valid = static_cast<int>(a.S - nfull * G);
-      if (valid > 0 && nfull >= q0 && nfull < q1 && ((nfull - q0) & (a.lanes - 1)) == lane)
-        lane_tail_group<N, F, PREC>(rk0, rk1, pu, f, static_cast<uint32_t>(nfull), valid, acc);
-    }
+    f.fx = fx;
   }
+  typename FxOf<F, PREC>::Acc acc;
+  sample_unit<N, F, PREC>(a, rk0, rk1, f, p, t, split, lane, acc);
+  s1 = acc.sum1();
+  s2 = acc.sum2();
 }
 
 // Reduce (s1, s2) over the `lanes` threads of each unit-split, in a fixed
@@ -480,13 +527,20 @@ scan_kernel(const __grid_constant__ ScanArgs a) {
   extern __shared__ double smem[];
   __shared__ double red[64];
   __shared__ float dimc[3 * ZMC_MAX_N];
+  const int64_t* fx = nullptr;
+  if constexpr (FxOf<F, PREC>::kTable != kFxNone) {
+    __shared__ int64_t fx_table[FxOf<F, PREC>::kEntries];
+    FxOf<F, PREC>::fill(fx_table);
+    if (!a.stage_smem) __syncthreads();  // else stage_lists ends with one
+    fx = fx_table;
+  }
   const void* table = stage_lists<N, F>(a, smem, dimc);
   const int lane = threadIdx.x & (a.lanes - 1);
   const int64_t us = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> a.lanes_log2) +
                      (threadIdx.x >> a.lanes_log2);
-  LaneAcc<PREC> acc;
-  if (us < a.n_us) unit_split_lane<N, F, PREC>(a, a.rk0, a.rk1, table, dimc, us, lane, acc);
-  double s1 = acc.sum1(), s2 = acc.sum2();
+  double s1 = 0.0, s2 = 0.0;
+  if (us < a.n_us)
+    unit_split_lane<N, F, PREC>(a, a.rk0, a.rk1, table, dimc, fx, us, lane, s1, s2);
   reduce_unit_split(a, s1, s2, red);
   if (lane == 0 && us < a.n_us && ZMC_CHECK(a.dbg, us >= 0, kDbgPartialSlot, us)) {
     a.partial[2 * us] = s1;
@@ -497,7 +551,7 @@ scan_kernel(const __grid_constant__ ScanArgs a) {
 #ifndef __CUDACC_RTC__
 template <int N, class F, int PREC>
 int launch_scan(const ScanArgs& a, int block, int64_t grid, size_t smem, void* stream) {
-  if (smem > 48 * 1024) {
+  if (smem + FxOf<F, PREC>::kStaticBytes + 1024 > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(scan_kernel<N, F, PREC>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));

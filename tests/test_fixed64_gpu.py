@@ -1,0 +1,106 @@
+"""FP64 scans whose parameters lie inside, at the edge of and outside the range of the
+fixed-point integrands, in one grid, against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import oracle
+from paper_1910_01965_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+PHASE_X = [0.0, -0.0, 5e-324, -1e-300, 1.7e-5, -3.25, 700.0, 2.0 ** 19, 1048575.5, -2.0 ** 20,
+           3e6, 1e9]
+BAD_X = [np.inf, -np.inf, np.nan, 1e307]
+
+
+@pytest.fixture(scope="module")
+def zmc():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1910_01965_gb300 import zmc as z
+    z.load()
+    return z
+
+
+def _run(z, gid, N, lo, hi, lists, S, T=2, seed=3, tiles=(0, 0, 0)):
+    lens = [len(v) for v in lists]
+    vals = np.concatenate(lists)
+    got, _ = z.scan(gid, N, lo, hi, lens, vals, S, T, seed, precision=z.ZMC_FP64,
+                    want_sums=True, tiles=tiles)
+    ref = oracle.default().scan(gid, N, lo, hi, lens, vals, S, T, seed, want_sums=True)
+    return got, ref
+
+
+def _compare(got, ref, N, lo, hi, S, phase):
+    """1e-12 of scale, plus what FP64 keeps of the phase: the oracle rounds y and
+    each product, N 2^-52 of the largest |phase| (one row per grid point)."""
+    V = float(np.prod(np.asarray(hi) - np.asarray(lo)))
+    R = V * np.sqrt(np.mean(ref["s2"], axis=1) / S)
+    tol = 1e-12 * np.maximum(np.abs(ref["mean"]), R) + V * N * 2.0 ** -52 * phase
+    ok = np.abs(got["mean"] - ref["mean"]) <= tol
+    nan = np.isnan(ref["mean"])
+    assert np.all(np.isnan(got["mean"]) == nan)
+    assert np.all(ok | nan), np.flatnonzero(~(ok | nan))
+
+
+@pytest.mark.parametrize("S,tiles", [(1, (0, 0, 0)), (7, (0, 0, 0)), (1003, (0, 0, 0)),
+                                     (1003, (2, 3, 64)), (333, (64, 1, 128))])
+@pytest.mark.parametrize("gid", [wl.G_COSPROD, wl.G_OSC01, wl.G_SINSUM])
+@pytest.mark.parametrize("N", [1, 2, 5])
+def test_phase_ranges(zmc, gid, N, S, tiles):
+    x = np.array(PHASE_X + BAD_X)
+    lists = [x] + [np.array([0.75])] * (N - 1)
+    lo, hi = np.full(N, -1.25), np.full(N, 2.0)
+    got, ref = _run(zmc, gid, N, lo, hi, lists, S, tiles=tiles)
+    with np.errstate(over="ignore"):
+        phase = 2.0 * (np.abs(np.where(np.isfinite(x), x, 0)) + 4 * N)
+    _compare(got, ref, N, lo, hi, S, phase)
+
+
+@pytest.mark.parametrize("lo,hi", [(-1.0, 1.0), (0.0, 1e-9), (1000.0, 1000.5), (-3.0, 8.0),
+                                   (1e5, 1e5 + 1), (-2e6, 1.0)])
+@pytest.mark.parametrize("gid", [wl.G_COSPROD, wl.G_OSC01, wl.G_SINSUM])
+def test_phase_boxes(zmc, gid, lo, hi):
+    N, S = 2, 501
+    x = np.array([0.5, -2.0, 30.0])
+    a, b = np.full(N, lo), np.full(N, hi)
+    got, ref = _run(zmc, gid, N, a, b, [x, np.array([1.5])], S)
+    m = max(abs(lo), abs(hi))
+    quad = 0.1 * m * m if gid == wl.G_OSC01 else 0.0
+    _compare(got, ref, N, a, b, S, N * (m * (np.abs(x) + 1.5) + quad))
+
+
+@pytest.mark.parametrize("N", [1, 3, 5, 8])
+@pytest.mark.parametrize("lo,hi", [(-1.0, 1.0), (0.0, 1e-9), (100.0, 101.5), (-5.6, 5.6),
+                                   (-30.0, 25.0)])
+def test_gauss_ranges(zmc, N, lo, hi):
+    """x inside the box, just within and beyond |x - y| = 15.9 / 2.83 and far out (g
+    underflows); far from the box the oracle's own exponent is rounded to
+    N 2^-53 q nats."""
+    mid, half = 0.5 * (lo + hi), 0.5 * (hi - lo)
+    x = np.array([mid, lo, hi, mid + 0.3, hi + 5.6 - 2 * half, hi + 5.7, hi + 9.0, hi + 60.0,
+                  np.inf, np.nan])
+    S, T = 1003, 2
+    a, b = np.full(N, lo), np.full(N, hi)
+    lists = [x] + [np.array([mid])] * (N - 1)
+    got, ref = _run(zmc, wl.G_GAUSS03, N, a, b, lists, S, T)
+    V = (hi - lo) ** N
+    R = V * np.sqrt(np.mean(ref["s2"], axis=1) / S)
+    far = np.maximum(np.abs(x - lo), np.abs(x - hi))
+    q = (far ** 2 + (N - 1) * half ** 2) / 0.18
+    tol = (1e-12 + N * 2.0 ** -51 * np.where(np.isfinite(q), q, 0)) * \
+        np.maximum(np.abs(ref["mean"]), R) + V * 1e-300
+    nan = np.isnan(ref["mean"])
+    assert np.all(np.isnan(got["mean"]) == nan)
+    assert np.all((np.abs(got["mean"] - ref["mean"]) <= tol) | nan)
+
+
+def test_unstaged_lists(zmc):
+    """More list values than shared memory takes (read from global memory)."""
+    r = np.random.default_rng(8)
+    x = r.uniform(0.5, 5.0, 5000)
+    x[::7] = 3e6
+    for gid, lo, hi in ((wl.G_COSPROD, 0.0, 1.0), (wl.G_GAUSS03, -1.0, 1.0)):
+        got, ref = _run(zmc, gid, 1, [lo], [hi], [x], 41)
+        _compare(got, ref, 1, [lo], [hi], 41, x * (gid == wl.G_COSPROD))
