@@ -42,14 +42,14 @@ int batch_blocks_per_sm(int precision, int block, size_t smem, int* out) {
 }
 
 constexpr int kBatchBlock = 256;
-// Sample groups per lane that bound one tile's work (tiles stay short next to
-// the whole batch, so the longest-first order balances the SMs).
+// Sample groups per lane that bound one tile's work (tiles stay
+// short next to the whole batch, so the longest-first order balances the SMs).
 constexpr int64_t kBatchGroupsPerLane = 1024;
 // Lanes per unit-split: the largest power of two <= 32 leaving each lane at
-// least this many sample groups (plain FP32 lane sums: 64).  Long lanes spend
-// less of their time in the FP64 epilogue on GB300's narrow FP64 unit:
-// measured, 512 against 64 makes the 2048 small scans of the serving mix 6 %
-// faster in one launch and leaves the uneven 256-scan batch unchanged.
+// least this many sample groups (plain FP32 lane sums: 64).  Long lanes spend less of their time in the FP64
+// epilogue on GB300's narrow FP64 unit: measured, 512 against 64 makes the 2048
+// small scans of the serving mix 6 % faster in one launch and leaves the uneven
+// 256-scan batch unchanged.
 #ifndef ZMC_BATCH_LANE_GROUPS
 #define ZMC_BATCH_LANE_GROUPS 512
 #endif
@@ -82,6 +82,11 @@ TilePlan plan_batch_scan(const zmc_scan_desc* d) {
   }
   tp.splits = static_cast<int>(std::min<int64_t>(std::max<int64_t>(splits, 1), Q));
   return tp;
+}
+
+int64_t batch_tiles(const zmc_scan_desc* d, int64_t count, const TilePlan& tp) {
+  const int64_t per_block = kBatchBlock / tp.lanes;
+  return (lane_groups_of(d, count, tp, nullptr, nullptr) + per_block - 1) / per_block;
 }
 
 struct PrecGroup {
@@ -185,8 +190,11 @@ int batch_create(const zmc_scan_desc* d, zmc_scan_out* o, int n, int flags, zmc_
     for (int k = 0; k < 6; ++k)
       if (ptrs[k] && !device_ptr(ptrs[k]))
         return fail(ZMC_EINVAL, "scan %d: a pointer is not device memory", i);
-    plans[i] = plan_batch_scan(&d[i]);
   }
+  int dev = 0, sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
+  for (int i = 0; i < n; ++i) plans[i] = plan_batch_scan(&d[i]);
 
   zmc_batch* b = new (std::nothrow) zmc_batch();
   if (!b) return fail(ZMC_ENOMEM, "host allocation failed");
@@ -196,13 +204,14 @@ int batch_create(const zmc_scan_desc* d, zmc_scan_out* o, int n, int flags, zmc_
   b->prefix.assign(n + 1, 0);
 
   // Per-scan unit-splits, tiles and partial-sum offsets.
-  std::vector<int64_t> n_us(n), ntiles(n), per_block(n);
+  std::vector<int64_t> n_us(n), n_lw(n), ntiles(n), per_block(n);
   std::vector<size_t> part_off(n);
   size_t part_bytes = 0;
   for (int i = 0; i < n; ++i) {
     n_us[i] = counts[i] * d[i].trials * plans[i].splits;
+    n_lw[i] = lane_groups_of(&d[i], counts[i], plans[i], nullptr, nullptr);
     per_block[i] = kBatchBlock / plans[i].lanes;
-    ntiles[i] = (n_us[i] + per_block[i] - 1) / per_block[i];
+    ntiles[i] = batch_tiles(&d[i], counts[i], plans[i]);
     part_off[i] = part_bytes;
     part_bytes += a256(static_cast<size_t>(n_us[i]) * 16);
     b->ntiles += ntiles[i];
@@ -255,25 +264,20 @@ int batch_create(const zmc_scan_desc* d, zmc_scan_out* o, int n, int flags, zmc_
   // tiles come first, each scan's tiles in order.
   std::vector<BatchTile> tiles;
   tiles.reserve(static_cast<size_t>(b->ntiles));
-  int dev = 0, sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
   for (int prec = 0; prec < 3; ++prec) {
     std::vector<int> order;
     for (int i = 0; i < n; ++i)
       if (d[i].precision == prec && ntiles[i] > 0) order.push_back(i);
     if (order.empty()) continue;
     // Longest tiles first: work per tile ~ unit-splits x samples per split x N.
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-      const int Gx = group_samples(d[x].N), Gy = group_samples(d[y].N);
-      const double cx = static_cast<double>(per_block[x]) * Gx *
-                        (((d[x].samples_per_point + Gx - 1) / Gx + plans[x].splits - 1) /
-                         plans[x].splits) * d[x].N;
-      const double cy = static_cast<double>(per_block[y]) * Gy *
-                        (((d[y].samples_per_point + Gy - 1) / Gy + plans[y].splits - 1) /
-                         plans[y].splits) * d[y].N;
-      return cx > cy;
-    });
+    auto tile_cost = [&](int x) {
+      const int Gx = group_samples(d[x].N);
+      return static_cast<double>(per_block[x]) * n_us[x] / n_lw[x] * Gx *
+             (((d[x].samples_per_point + Gx - 1) / Gx + plans[x].splits - 1) /
+              plans[x].splits) * d[x].N;
+    };
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int x, int y) { return tile_cost(x) > tile_cost(y); });
     PrecGroup g;
     g.precision = prec;
     g.tile_begin = static_cast<int64_t>(tiles.size());
@@ -281,8 +285,8 @@ int batch_create(const zmc_scan_desc* d, zmc_scan_out* o, int n, int flags, zmc_
       for (int64_t k = 0; k < ntiles[i]; ++k) {
         BatchTile t;
         t.scan = i;
-        t.first_us = k * per_block[i];
-        t.units = static_cast<int32_t>(std::min<int64_t>(per_block[i], n_us[i] - t.first_us));
+        t.first_w = k * per_block[i];
+        t.units = static_cast<int32_t>(std::min<int64_t>(per_block[i], n_lw[i] - t.first_w));
         tiles.push_back(t);
       }
       if (b->args[i].stage_smem)

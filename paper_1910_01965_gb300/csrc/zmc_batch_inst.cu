@@ -2,7 +2,7 @@
 // precision (compiled once per ZMC_INST_PREC).
 //
 // Many scans of different integrands, dimensions, grid sizes and sample counts
-// run in one launch.  The host cuts every scan into tiles — the unit-splits one
+// run in one launch.  The host cuts every scan into tiles — the lane groups one
 // block sums at once, all of one scan — and orders them longest first.  Each
 // resident block takes the next tile from a device counter (one atomicAdd by
 // thread 0, no waiting on other blocks), stages that scan's lists or constant
@@ -56,20 +56,9 @@ __device__ __noinline__ void batch_tile(const ScanArgs& a, const BatchTile& t, b
     rk0[r] = a.rk0[r];
     rk1[r] = a.rk1[r];
   }
-  const int lane = threadIdx.x & (a.lanes - 1);
-  const int local = threadIdx.x >> a.lanes_log2;
-  const bool active = local < t.units;
-  const int64_t us = t.first_us + local;
-  double s1 = 0.0, s2 = 0.0;
-  if (active)
-    unit_split_lane<N, F, PREC>(a, rk0, rk1, table, dimc,
-                                FxOf<F, PREC>::kTable == kFxExpTable ? fxe : fxc, us, lane, s1,
-                                s2);
-  reduce_unit_split(a, s1, s2, red);
-  if (lane == 0 && active && ZMC_CHECK(a.dbg, us >= 0 && us < a.n_us, kDbgPartialSlot, us)) {
-    a.partial[2 * us] = s1;
-    a.partial[2 * us + 1] = s2;
-  }
+  block_work<N, F, PREC>(a, rk0, rk1, table, dimc,
+                         FxOf<F, PREC>::kTable == kFxExpTable ? fxe : fxc, t.first_w, t.units,
+                         red);
 }
 
 #define ZMC_CASE_N(gid, F, n)                                                        \
@@ -85,7 +74,7 @@ template <int PREC>
 __global__ void __launch_bounds__(256, ZMC_BATCH_MIN_BLOCKS)
 batch_kernel(const __grid_constant__ BatchArgs b) {
   extern __shared__ double smem[];
-  __shared__ double red[64];
+  __shared__ double red[kReduceDoubles];
   __shared__ float dimc[3 * ZMC_MAX_N];
   __shared__ long long s_tile;
   const int64_t *fxc = nullptr, *fxe = nullptr;

@@ -34,6 +34,17 @@ enum {
   kDbgFinalize = 6      // a finalize index beyond its scan's points
 };
 
+// Constants of the FP32 field extraction, passed as arguments so that the
+// compiler does not fold them (field_value).
+struct FieldConst {
+  uint32_t mask = 0x7fffffu;     // 23 bits
+  uint32_t one = 0x3f800000u;    // 1.0f
+  uint32_t shl4 = 16;            // shift left by 4
+};
+
+// Trials of one grid point that the same lanes sample together, at most.
+constexpr int kMaxLaneTrials = 4;
+
 // Everything one launch of the sampling kernel needs, passed by value.
 // A "unit" is one (grid point, trial) pair; its S samples are cut into
 // `splits` contiguous ranges of sample groups, and each range (a
@@ -45,6 +56,8 @@ struct ScanArgs {
   int64_t ngroups;      // sample groups per unit: ceil(S / G)
   int64_t gps;          // sample groups per split: ceil(ngroups / splits)
   int64_t n_us;         // unit-splits: count * T * splits
+  int64_t n_lw;         // lane groups: one per unit-splits sampled together
+  int64_t lu4, lu2;     // lane groups of four and of two trials (they come first)
   int32_t T;
   int32_t M;
   int32_t splits;
@@ -62,6 +75,7 @@ struct ScanArgs {
   double hi[ZMC_MAX_N];
   uint32_t rk0[10];     // Philox round keys: key0 + r * W0
   uint32_t rk1[10];     // Philox round keys: key1 + r * W1
+  FieldConst field;
   double* partial;      // device, [n_us][2] FP64 (sum g, sum g^2)
   unsigned long long* dbg;  // device check words (ZMC_DEBUG builds), or null
 };
@@ -97,11 +111,11 @@ ScanLaunchFn scan_launcher(int precision, int integrand, int N);
 int finalize_launch(const FinalizeArgs& a, void* stream);
 
 // ------------------------------------------------------------- batches --
-// One tile = the unit-splits one block sums at once, all of one scan.
+// One tile = the lane groups one block sums at once, all of one scan.
 struct BatchTile {
-  int32_t scan;      // index into the batch's ScanArgs array
-  int32_t units;     // unit-splits in this tile (<= block / lanes)
-  int64_t first_us;  // first unit-split of the tile
+  int32_t scan;     // index into the batch's ScanArgs array
+  int32_t units;    // lane groups in this tile (<= block / lanes)
+  int64_t first_w;  // first lane group of the tile
 };
 
 struct BatchArgs {

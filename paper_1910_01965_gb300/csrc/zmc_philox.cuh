@@ -9,7 +9,11 @@
 // Because three of the four counter words are fixed per unit, round 1's
 // second multiply and round 2's first multiply do not depend on j.  They are
 // computed once per unit (PhiloxUnit) and the per-call work drops from 20 to
-// 18 multiplies.  The outputs are bit-identical to the plain ten rounds.
+// 18 multiplies.  Round 2's second and round 3's first multiply do not depend
+// on the trial t: a lane that samples B trials of a point together computes
+// them once (PhiloxShared), which leaves 15 + 2/B multiplies per call with the
+// first one carried along.  The outputs are bit-identical to the plain ten
+// rounds.
 #pragma once
 
 #include <cstdint>
@@ -61,25 +65,43 @@ __device__ __forceinline__ void add64(uint32_t& lo, uint32_t& hi, uint32_t alo, 
       : "+r"(lo), "+r"(hi) : "r"(alo), "r"(ahi));
 }
 
-// Four words of the call whose round-1 product M0 * j is (H0:L0).  A lane
-// walking j in fixed strides carries this product with one 64-bit add per
-// call instead of a 32x32->64 multiply.
-__device__ __forceinline__ void philox_call_pre(const PhiloxUnit& u,
-                                                const uint32_t* __restrict__ rk0,
-                                                const uint32_t* __restrict__ rk1,
-                                                uint32_t H0, uint32_t L0, uint32_t* out) {
+// The part of a call that is the same for every trial of a grid point, from the
+// round-1 product M0 * j = (H0:L0): round 2's M1 product and round 3's M0 product
+// (b0 does not depend on the trial).  A lane that samples several trials of a
+// point computes it once for all of them; and walking j in fixed strides it
+// carries M0 * j with one 64-bit add per call instead of a 32x32->64 multiply.
+struct PhiloxShared {
+  uint32_t L0;        // low word of M0 * j
+  uint32_t L1;        // round-2 output word 1
+  uint32_t hi0, lo0;  // round 3's M0 product
+};
+
+__device__ __forceinline__ PhiloxShared philox_shared(uint32_t a2, uint32_t b0, uint32_t H0,
+                                                      uint32_t L0) {
+  PhiloxShared s;
+  s.L0 = L0;
   // Round 1: words become (c0, c1, H0 ^ p_hi ^ k1, L0).
-  const uint32_t c2 = H0 ^ u.a2;
+  const uint32_t c2 = H0 ^ a2;
   // Round 2: only mulhilo(M1, c2) depends on j.
-  uint32_t H1, L1;
-  mulhilo32(kPhiloxM1, c2, H1, L1);
-  uint32_t x0 = H1 ^ u.b0;
-  uint32_t x1 = L1;
-  uint32_t x2 = L0 ^ u.b1;
-  uint32_t x3 = u.b2;
+  uint32_t H1;
+  mulhilo32(kPhiloxM1, c2, H1, s.L1);
+  mulhilo32(kPhiloxM0, H1 ^ b0, s.hi0, s.lo0);
+  return s;
+}
+
+// Four words of the call from its shared part and the trial's b1, b2.
+__device__ __forceinline__ void philox_finish(const PhiloxShared& s, uint32_t b1, uint32_t b2,
+                                              const uint32_t* __restrict__ rk0,
+                                              const uint32_t* __restrict__ rk1, uint32_t* out) {
+  uint32_t hi1, lo1;
+  mulhilo32(kPhiloxM1, s.L0 ^ b1, hi1, lo1);
+  uint32_t x0 = hi1 ^ s.L1 ^ rk0[2];
+  uint32_t x1 = lo1;
+  uint32_t x2 = s.hi0 ^ b2 ^ rk1[2];
+  uint32_t x3 = s.lo0;
 #pragma unroll
-  for (int r = 2; r < 10; ++r) {
-    uint32_t hi0, lo0, hi1, lo1;
+  for (int r = 3; r < 10; ++r) {
+    uint32_t hi0, lo0;
     mulhilo32(kPhiloxM0, x0, hi0, lo0);
     mulhilo32(kPhiloxM1, x2, hi1, lo1);
     const uint32_t n0 = hi1 ^ x1 ^ rk0[r];
@@ -102,7 +124,7 @@ __device__ __forceinline__ void philox_call(const PhiloxUnit& u,
                                             uint32_t j, uint32_t* out) {
   uint32_t H0, L0;
   mulhilo32(kPhiloxM0, j, H0, L0);
-  philox_call_pre(u, rk0, rk1, H0, L0, out);
+  philox_finish(philox_shared(u.a2, u.b0, H0, L0), u.b1, u.b2, rk0, rk1, out);
 }
 
 // Round-1 products M0 * j for j = j0, j0 + stride, j0 + 2 stride, ...

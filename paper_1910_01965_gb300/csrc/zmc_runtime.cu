@@ -266,6 +266,44 @@ TilePlan plan_tiles(int N, int64_t S, int T, int64_t count, int sm_count,
   return tp;
 }
 
+int max_lane_trials(const zmc_scan_desc* d) {
+  if (d->precision == ZMC_FP64 || d->integrand_id == ZMC_G_CONST) return 1;
+  return d->trials >= 4 ? 4 : d->trials >= 2 ? 2 : 1;
+}
+
+// Trials per lane: 4, 2 or 1, whichever ends first by this model.  Blocks are
+// spread over the SMs in rounds (one 256-thread block keeps an SM busy), those
+// with more trials first; a block of 4 (2) trials takes 3.74 (1.92) times as long
+// as one of a single trial, having shared part of its Philox calls.  Measured on
+// the Gaussian at N = 4 (T = 4, 2^14 samples, 32 lanes): one round of blocks
+// takes 46 us with one trial and 165-172 us with four, so 1000 points (125
+// blocks of four trials on 152 SMs) run in 185 against 189 us, 1500 points (187
+// blocks, two rounds) in 345 against 235 us, 10^5 points in 13.5 against 14.2 ms.
+static int plan_lane_trials(const zmc_scan_desc* d, int64_t count, const TilePlan& tp, int sm) {
+  int best = 1;
+  double best_cost = 0.0;
+  sm = std::max(1, sm);
+  for (int b = 1; b <= max_lane_trials(d); b <<= 1) {
+    TilePlan t = tp;
+    t.trials = b;
+    int64_t lu4 = 0, lu2 = 0;
+    const int64_t lw = lane_groups_of(d, count, t, &lu4, &lu2);
+    const double per_block = static_cast<double>(tp.block / tp.lanes);
+    const double n4 = lu4 / per_block, n2 = lu2 / per_block, n1 = (lw - lu4 - lu2) / per_block;
+    const double first = n4 > 0 ? 3.74 : n2 > 0 ? 1.92 : 1.0;
+    const double rounds = std::ceil((n4 > 0 ? n4 : n2 > 0 ? n2 : n1) / sm) * first;
+    const double all = (3.74 * n4 + 1.92 * n2 + n1) / sm;
+    const double cost = n1 > 0 && first > 1.0 ? std::max(rounds, all + 0.5)
+                        : n2 > 0 && n4 > 0    ? std::max(rounds, all + 1.0)
+                                              : rounds;
+    if (b == 1 || cost < best_cost) {
+      best = b;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 static size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 // ------------------------------------------------------------- chunking --
@@ -316,7 +354,7 @@ ScanLayout layout_for(const zmc_scan_desc* d, int64_t count, const TilePlan& tp)
   return L;
 }
 
-TilePlan plan_with(const zmc_scan_desc* d, int64_t count, int sm, int tps) {
+static TilePlan plan_sums(const zmc_scan_desc* d, int64_t count, int sm, int tps) {
   // A class entry recorded by the autotuner, when the caller leaves tiles open.
   int tl = 0, tb = 0, tg = 0;
   if (!d->tile_lanes && !d->tile_splits && !d->tile_block &&
@@ -339,6 +377,12 @@ TilePlan plan_with(const zmc_scan_desc* d, int64_t count, int sm, int tps) {
   }
   return plan_tiles(d->N, d->samples_per_point, d->trials, count, sm, tps, d->tile_lanes,
                     d->tile_splits, d->tile_block, d->precision);
+}
+
+TilePlan plan_with(const zmc_scan_desc* d, int64_t count, int sm, int tps) {
+  TilePlan tp = plan_sums(d, count, sm, tps);
+  tp.trials = plan_lane_trials(d, count, tp, sm);
+  return tp;
 }
 
 int plan_for(const zmc_scan_desc* d, int64_t count, TilePlan* tp) {
@@ -364,6 +408,17 @@ static void fill_round_keys(uint64_t seed, uint32_t* rk0, uint32_t* rk1) {
   }
 }
 
+int64_t lane_groups_of(const zmc_scan_desc* d, int64_t count, const TilePlan& tp, int64_t* lu4,
+                       int64_t* lu2) {
+  const int64_t T = d->trials;
+  const int64_t n4 = tp.trials >= 4 ? T / 4 : 0;
+  const int64_t n2 = tp.trials >= 2 ? (T - 4 * n4) / 2 : 0;
+  const int64_t n1 = T - 4 * n4 - 2 * n2;
+  if (lu4) *lu4 = count * n4 * tp.splits;
+  if (lu2) *lu2 = count * n2 * tp.splits;
+  return count * (n4 + n2 + n1) * tp.splits;
+}
+
 double box_volume(const zmc_scan_desc* d) {
   double V = 1.0;
   for (int k = 0; k < d->N; ++k) V *= d->hi[k] - d->lo[k];
@@ -372,7 +427,7 @@ double box_volume(const zmc_scan_desc* d) {
 
 void fill_scan_args(const zmc_scan_desc* d, int64_t count, const TilePlan& tp,
                     const double* vals_dev, double* partial_dev, ScanArgs* a) {
-  std::memset(a, 0, sizeof(*a));
+  *a = ScanArgs();
   const int G = group_samples(d->N);
   a->first = d->first_index;
   a->count = count;
@@ -383,6 +438,7 @@ void fill_scan_args(const zmc_scan_desc* d, int64_t count, const TilePlan& tp,
   a->T = d->trials;
   a->M = d->M;
   a->n_us = count * d->trials * tp.splits;
+  a->n_lw = lane_groups_of(d, count, tp, &a->lu4, &a->lu2);
   a->lanes = tp.lanes;
   int l2 = 0;
   while ((1 << l2) < tp.lanes) ++l2;
@@ -402,6 +458,7 @@ void fill_scan_args(const zmc_scan_desc* d, int64_t count, const TilePlan& tp,
     a->hi[k] = d->hi[k];
   }
   fill_round_keys(d->seed, a->rk0, a->rk1);
+  a->field = FieldConst();
   a->partial = partial_dev;
   a->dbg = debug_words();
   a->gid = d->integrand_id;
@@ -413,7 +470,7 @@ int launch_scan_args(const zmc_scan_desc* d, const ScanArgs& a, const TilePlan& 
   if (a.n_us == 0) return ZMC_OK;
   if (is_user_integrand(d->integrand_id)) {
     const int64_t per_block = tp.block / tp.lanes;
-    const int64_t grid = (a.n_us + per_block - 1) / per_block;
+    const int64_t grid = (a.n_lw + per_block - 1) / per_block;
     if (grid > 0x7fffffffLL) return fail(ZMC_EINVAL, "launch grid too large (%lld)", (long long)grid);
     const size_t smem = a.stage_smem ? static_cast<size_t>(a.nvals) * sizeof(double) : 0;
     return user_launch(d, a, tp.block, grid, smem, stream);
@@ -421,7 +478,7 @@ int launch_scan_args(const zmc_scan_desc* d, const ScanArgs& a, const TilePlan& 
   ScanLaunchFn fn = scan_launcher(d->precision, d->integrand_id, d->N);
   if (!fn) return fail(ZMC_ENOTFOUND, "no kernel for integrand %d, N %d", d->integrand_id, d->N);
   const int64_t per_block = tp.block / tp.lanes;
-  const int64_t grid = (a.n_us + per_block - 1) / per_block;
+  const int64_t grid = (a.n_lw + per_block - 1) / per_block;
   if (grid > 0x7fffffffLL) return fail(ZMC_EINVAL, "launch grid too large (%lld)", (long long)grid);
   const size_t smem = a.stage_smem ? static_cast<size_t>(a.nvals) * sizeof(double) : 0;
   int e = fn(a, tp.block, grid, smem, stream);

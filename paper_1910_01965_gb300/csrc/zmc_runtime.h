@@ -14,6 +14,7 @@ struct TilePlan {
   int lanes = 32;   // threads summing one unit-split (power of two)
   int splits = 1;   // sample ranges per (point, trial) unit
   int block = 256;  // threads per block
+  int trials = 1;   // trials of a point that the same lanes sample (1, 2, 4)
 };
 
 // Byte offsets of each region inside one scan's device scratch.  The slice
@@ -53,6 +54,15 @@ void tune_ensure_loaded();
 bool tune_find(int prec, int gid, int N, int64_t S, int* lanes, int* block, int* gpl);
 ScanLayout layout_for(const zmc_scan_desc* d, int64_t count, const TilePlan& tp);
 int64_t chunk_points_for(const zmc_scan_desc* d, int64_t count, const TilePlan& tp);
+// The most trials of a point that one lane of this scan's kernel samples.
+int max_lane_trials(const zmc_scan_desc* d);
+// The plan of a batched or served scan, and the number of tiles of `count` points.
+TilePlan plan_batch_scan(const zmc_scan_desc* d);
+int64_t batch_tiles(const zmc_scan_desc* d, int64_t count, const TilePlan& tp);
+// Lane groups of a launch over `count` points (and how many of them take four
+// and two trials, may be null).
+int64_t lane_groups_of(const zmc_scan_desc* d, int64_t count, const TilePlan& tp, int64_t* lu4,
+                       int64_t* lu2);
 double box_volume(const zmc_scan_desc* d);
 void fill_scan_args(const zmc_scan_desc* d, int64_t count, const TilePlan& tp,
                     const double* vals_dev, double* partial_dev, ScanArgs* a);

@@ -4,7 +4,9 @@
 // (grid point p, trial t) sums g over its S samples.  The paper gives each
 // grid point to one GPU thread that loops over all samples (Sec. 2, Fig. 1);
 // here a unit's samples are cut into `splits` ranges and each range is summed
-// by `lanes` threads, so that a grid of any shape fills all SMs.  Lane sums
+// by `lanes` threads, so that a grid of any shape fills all SMs.  Up to four
+// trials of a point are summed by the same threads, which share a part of their
+// Philox calls.  Lane sums
 // are reduced with warp shuffles and, for ranges wider than a warp, through
 // shared memory, in a fixed order; each range writes one FP64 (sum g,
 // sum g^2) pair.  The finalize kernel (K2) adds the ranges in order and forms
@@ -266,72 +268,90 @@ __device__ __forceinline__ const void* stage_lists(const ScanArgs& a, double* sm
 // come from the group's fields g*N .. g*N + N - 1 (field e is field e mod 5
 // of the group's call e / 5).
 template <int N, class F>
-__device__ __forceinline__ auto eval_sample(const F& f, const uint32_t* r, int g) {
+__device__ __forceinline__ auto eval_sample(const F& f, const FieldConst& fc,
+                                            const uint32_t* r, int g) {
   typename F::unit_t u[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
     const int e = g * N + k;
-    u[k] = field_unit<typename F::unit_t>(
-        field23(r + 4 * (e / kFieldsPerCall), e % kFieldsPerCall));
+    u[k] = field_value<typename F::unit_t>(fc, r + 4 * (e / kFieldsPerCall),
+                                           e % kFieldsPerCall);
   }
   return f.eval(u);
 }
 
-// Sum over the sample groups [q, q_end) with stride `step` (one lane).
+// A lane samples this many trials of one grid point together at most (they
+// share a part of every Philox call); the FP64 kernels, bound elsewhere, and the
+// constant integrand, which draws nothing, take one.
+template <class F, int PREC>
+constexpr int max_trials() {
+  return PREC == kPrecFP64 || !F::kUsesSamples ? 1 : kMaxLaneTrials;
+}
+
+// Sums over the sample groups [q, q_end) with stride `step` (one lane) of B
+// trials, trial u of them with the Philox constants b1[u], b2[u].
 //
-// Order of the compensated additions (the same for every blocking choice
-// below, so the single-scan and batched kernels agree bit for bit): with
+// Order of the compensated additions of a trial (the same for every blocking
+// choice below, so that the results do not depend on how many trials a lane
+// takes, and the single-scan and batched kernels agree bit for bit): with
 // G = 5, each group's five samples enter in one step (LaneAcc::add_group), in
 // group order; with G = 1, consecutive groups are paired and a last unpaired
 // group enters alone.
-template <int N, class F, int PREC, class Acc>
+template <int N, class F, int PREC, int B, class Acc>
 __device__ __forceinline__ void lane_groups(const uint32_t* __restrict__ rk0,
-                                            const uint32_t* __restrict__ rk1,
-                                            const PhiloxUnit& pu, const F& f, uint32_t q,
-                                            uint32_t q_end, uint32_t step,
-                                            Acc& acc) {
+                                            const uint32_t* __restrict__ rk1, uint32_t a2,
+                                            uint32_t b0, const uint32_t (&b1)[B],
+                                            const uint32_t (&b2)[B], const F& f,
+                                            const FieldConst& fc, uint32_t q, uint32_t q_end,
+                                            uint32_t step, Acc (&acc)[B]) {
   constexpr int G = group_samples(N);
   constexpr int C = group_calls(N);
   // Groups per loop block: about kCallsInFlight independent Philox chains
-  // per lane (a group of C calls already has C).  The FP64 path is bound by
-  // its FP64 arithmetic, not by the stream: one group at a time.
+  // per lane (a group of C calls of B trials already has C B).  The FP64 path
+  // draws one group at a time.
 #ifdef ZMC_CALLS_IN_FLIGHT
   constexpr int kCalls = PREC == kPrecFP64 ? 1 : ZMC_CALLS_IN_FLIGHT;
 #else
   constexpr int kCalls = PREC == kPrecFP64 ? 1 : F::kCallsInFlight;
 #endif
-  constexpr int kBlock = kCalls / C > 1 ? kCalls / C : 1;
+  constexpr int kBlock = kCalls / (C * B) > 1 ? kCalls / (C * B) : 1;
+  using T = decltype(eval_sample<N>(f, fc, static_cast<const uint32_t*>(nullptr), 0));
   // M0 * j for the lane's calls, carried along by 64-bit adds: call c of
   // group q has j = q C + c; the product for q C advances with the lane's
   // stride and call c adds the constant M0 c to it.
   StridedProduct sp;
   sp.init(q * C, step * C);
-  auto call = [&](int c, uint32_t* out) {
+  // Words of call c of the current group, every trial: out[u][4 * at ..].
+  auto call = [&](int c, auto& out, int at) {
     uint32_t H, L;
     sp.at(c, H, L);
-    philox_call_pre(pu, rk0, rk1, H, L, out);
+    const PhiloxShared sh = philox_shared(a2, b0, H, L);
+#pragma unroll
+    for (int u = 0; u < B; ++u) philox_finish(sh, b1[u], b2[u], rk0, rk1, &out[u][4 * at]);
   };
   // Draw the words of V consecutive groups of this lane.
   auto draw = [&](auto& r) {
     constexpr int V = sizeof(r) / sizeof(r[0]);
 #pragma unroll
-    for (int u = 0; u < V; ++u) {
+    for (int i = 0; i < V; ++i) {
 #pragma unroll
-      for (int c = 0; c < C; ++c) call(c, &r[u][4 * c]);
+      for (int c = 0; c < C; ++c) call(c, r[i], c);
       sp.advance();
     }
   };
   if constexpr (G > 1) {
     constexpr int U = kBlock;
-    using T = decltype(eval_sample<N>(f, static_cast<const uint32_t*>(nullptr), 0));
     auto consume = [&](const auto& r) {
       constexpr int V = sizeof(r) / sizeof(r[0]);
 #pragma unroll
-      for (int u = 0; u < V; ++u) {
-        T v[G];
+      for (int i = 0; i < V; ++i) {
 #pragma unroll
-        for (int g = 0; g < G; ++g) v[g] = eval_sample<N>(f, r[u], g);
-        acc.template add_group<G>(v);
+        for (int u = 0; u < B; ++u) {
+          T v[G];
+#pragma unroll
+          for (int g = 0; g < G; ++g) v[g] = eval_sample<N>(f, fc, r[i][u], g);
+          acc[u].template add_group<G>(v);
+        }
       }
     };
     if constexpr (U == 1 && C > 2) {
@@ -339,28 +359,30 @@ __device__ __forceinline__ void lane_groups(const uint32_t* __restrict__ rk0,
       // sample that reads it, so a call's words die once its last sample is
       // evaluated (fewer live registers than drawing all C calls first).
       for (; q < q_end; q += step) {
-        uint32_t r[4 * C];
-        T v[G];
+        uint32_t r[B][4 * C];
+        T v[B][G];
 #pragma unroll
         for (int g = 0; g < G; ++g) {
           const int c0 = g == 0 ? 0 : (g * N - 1) / kFieldsPerCall + 1;
           const int c1 = (g * N + N - 1) / kFieldsPerCall;
 #pragma unroll
-          for (int c = c0; c <= c1; ++c) call(c, &r[4 * c]);
-          v[g] = eval_sample<N>(f, r, g);
+          for (int c = c0; c <= c1; ++c) call(c, r, c);
+#pragma unroll
+          for (int u = 0; u < B; ++u) v[u][g] = eval_sample<N>(f, fc, r[u], g);
         }
-        acc.template add_group<G>(v);
+#pragma unroll
+        for (int u = 0; u < B; ++u) acc[u].template add_group<G>(v[u]);
         sp.advance();
       }
     } else {
       for (; q + (U - 1) * step < q_end; q += U * step) {
-        uint32_t r[U][4 * C];
+        uint32_t r[U][B][4 * C];
         draw(r);
         consume(r);
       }
       if constexpr (U > 1) {
         for (; q < q_end; q += step) {
-          uint32_t r[1][4 * C];
+          uint32_t r[1][B][4 * C];
           draw(r);
           consume(r);
         }
@@ -372,26 +394,29 @@ __device__ __forceinline__ void lane_groups(const uint32_t* __restrict__ rk0,
     auto consume = [&](const auto& r) {
       constexpr int V = sizeof(r) / sizeof(r[0]);
 #pragma unroll
-      for (int u = 0; u < V; u += 2)
-        acc.add2(eval_sample<N>(f, r[u], 0), eval_sample<N>(f, r[u + 1], 0));
+      for (int i = 0; i < V; i += 2)
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          acc[u].add2(eval_sample<N>(f, fc, r[i][u], 0), eval_sample<N>(f, fc, r[i + 1][u], 0));
     };
     for (; q + (U - 1) * step < q_end; q += U * step) {
-      uint32_t r[U][4 * C];
+      uint32_t r[U][B][4 * C];
       draw(r);
       consume(r);
     }
     // Fewer than U groups left: pairs, then a single group.
     if constexpr (U > 2) {
       for (; q + step < q_end; q += 2 * step) {
-        uint32_t r[2][4 * C];
+        uint32_t r[2][B][4 * C];
         draw(r);
         consume(r);
       }
     }
     if (q < q_end) {
-      uint32_t r[1][4 * C];
+      uint32_t r[1][B][4 * C];
       draw(r);
-      acc.add(eval_sample<N>(f, r[0], 0));
+#pragma unroll
+      for (int u = 0; u < B; ++u) acc[u].add(eval_sample<N>(f, fc, r[0][u], 0));
     }
   }
 }
@@ -401,8 +426,8 @@ __device__ __forceinline__ void lane_groups(const uint32_t* __restrict__ rk0,
 template <int N, class F, class Acc>
 __device__ __forceinline__ void lane_tail_group(const uint32_t* __restrict__ rk0,
                                                 const uint32_t* __restrict__ rk1,
-                                                const PhiloxUnit& pu, const F& f, uint32_t q,
-                                                int valid, Acc& acc) {
+                                                const PhiloxUnit& pu, const F& f,
+                                                const FieldConst& fc, uint32_t q, int valid, Acc& acc) {
   constexpr int G = group_samples(N);
   constexpr int C = group_calls(N);
   uint32_t r[4 * C];
@@ -410,15 +435,18 @@ __device__ __forceinline__ void lane_tail_group(const uint32_t* __restrict__ rk0
   for (int c = 0; c < C; ++c) philox_call(pu, rk0, rk1, q * C + c, &r[4 * c]);
 #pragma unroll
   for (int g = 0; g < G; ++g)
-    if (g < valid) acc.add(eval_sample<N>(f, r, g));
+    if (g < valid) acc.add(eval_sample<N>(f, fc, r, g));
 }
 
-// Sums of one lane over its part of unit-split `split` of unit (p, t).
-template <int N, class F, int PREC, class Acc>
-__device__ __forceinline__ void sample_unit(const ScanArgs& a, const uint32_t* rk0,
-                                            const uint32_t* rk1, const F& f, int64_t p,
-                                            uint32_t t, int64_t split, int lane, Acc& acc) {
+// Sums of one lane over its part of split `split` of trials t .. t + B - 1 of
+// point p.
+template <int N, class F, int PREC, int B>
+__device__ __forceinline__ void sample_trials(const ScanArgs& a, const uint32_t* rk0,
+                                              const uint32_t* rk1, const F& f, int64_t p,
+                                              uint32_t t, int64_t split, int lane, double* s1,
+                                              double* s2) {
   constexpr int G = group_samples(N);
+  typename FxOf<F, PREC>::Acc acc[B];
   const int64_t q0 = split * a.gps;
   const int64_t q1 = min(q0 + a.gps, a.ngroups);
   if constexpr (!F::kUsesSamples) {
@@ -426,106 +454,240 @@ __device__ __forceinline__ void sample_unit(const ScanArgs& a, const uint32_t* r
     for (int64_t q = q0 + lane; q < q1; q += a.lanes) {
       const int64_t left = a.S - q * G;
       const int cnt = left < G ? static_cast<int>(left) : G;
-      for (int g = 0; g < cnt; ++g) acc.add(f.eval(nullptr));
+      for (int g = 0; g < cnt; ++g) acc[0].add(f.eval(nullptr));
     }
   } else {
-    const PhiloxUnit pu = philox_unit(rk0, rk1, static_cast<uint64_t>(p), t);
+    PhiloxUnit pu[B];
+    uint32_t b1[B], b2[B];
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      pu[u] = philox_unit(rk0, rk1, static_cast<uint64_t>(p), t + u);
+      b1[u] = pu[u].b1;
+      b2[u] = pu[u].b2;
+    }
     const int64_t nfull = a.S / G;
     const int64_t qf = min(q1, nfull);
     if (q0 + lane < qf)
-      lane_groups<N, F, PREC>(rk0, rk1, pu, f, static_cast<uint32_t>(q0 + lane),
-                              static_cast<uint32_t>(qf), static_cast<uint32_t>(a.lanes),
-                              acc);
+      lane_groups<N, F, PREC, B>(rk0, rk1, pu[0].a2, pu[0].b0, b1, b2, f, a.field,
+                                 static_cast<uint32_t>(q0 + lane), static_cast<uint32_t>(qf),
+                                 static_cast<uint32_t>(a.lanes), acc);
     if (G > 1) {
       const int valid = static_cast<int>(a.S - nfull * G);
       if (valid > 0 && nfull >= q0 && nfull < q1 && ((nfull - q0) & (a.lanes - 1)) == lane)
-        lane_tail_group<N, F>(rk0, rk1, pu, f, static_cast<uint32_t>(nfull), valid, acc);
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          lane_tail_group<N, F>(rk0, rk1, pu[u], f, a.field, static_cast<uint32_t>(nfull), valid,
+                                acc[u]);
     }
+  }
+#pragma unroll
+  for (int u = 0; u < B; ++u) {
+    s1[u] = acc[u].sum1();
+    s2[u] = acc[u].sum2();
   }
 }
 
-// The same with an FP64 functor for parameters outside a fixed-point functor's
-// range.  Not inlined, so that it takes no registers from the usual path.
+// The same for one trial with an FP64 functor, for parameters outside a
+// fixed-point functor's range.  Not inlined, so that it takes no registers from
+// the usual path.
 template <int N, class F, int PREC>
 __device__ __noinline__ void sample_unit_wide(const ScanArgs& a, const void* table, int64_t p,
-                                              uint32_t t, int64_t split, int lane, double& s1,
-                                              double& s2) {
+                                              uint32_t t, int64_t split, int lane, double* s1,
+                                              double* s2) {
   F f{};
   load_params<N>(a, table, static_cast<const float*>(nullptr), p, f);
-  LaneAcc<PREC> acc;
-  sample_unit<N, F, PREC>(a, a.rk0, a.rk1, f, p, t, split, lane, acc);
-  s1 = acc.sum1();
-  s2 = acc.sum2();
+  sample_trials<N, F, PREC, 1>(a, a.rk0, a.rk1, f, p, t, split, lane, s1, s2);
 }
 
-// Work of one lane for unit-split `us`: decode, prepare, sample, sum.
-// rk0/rk1 are the ten Philox round keys (parameter space in the single-scan
-// kernel, registers in the batched one); fx the fixed-point functors' table.
+// The work of the `lanes` threads of lane group w: `trials` trials from t on of
+// grid point first + lp, sample split `split`.  The groups with four trials come
+// first, then those with two, then single trials (lu4, lu2: how many).
+struct LaneWork {
+  int64_t lp, split;
+  uint32_t t;
+  int trials;
+};
+
+__device__ __forceinline__ int lane_trials(const ScanArgs& a, int64_t w) {
+  return w < a.lu4 ? 4 : w < a.lu4 + a.lu2 ? 2 : 1;
+}
+
+template <int MAXB>
+__device__ __forceinline__ LaneWork lane_work(const ScanArgs& a, int64_t w) {
+  int per = a.T;  // lane groups of this size per point and split
+  LaneWork k;
+  k.trials = 1;
+  k.t = 0;
+  if constexpr (MAXB > 1) {
+    k.trials = lane_trials(a, w);
+    if (k.trials == 4) {
+      per = a.T >> 2;
+    } else if (k.trials == 2) {
+      w -= a.lu4;
+      k.t = a.lu4 ? a.T & ~3 : 0;
+      per = (a.T - static_cast<int>(k.t)) >> 1;
+    } else {
+      w -= a.lu4 + a.lu2;
+      k.t = a.lu2 ? a.T & ~1 : a.lu4 ? a.T & ~3 : 0;
+      per = a.T - static_cast<int>(k.t);
+    }
+  }
+  const int64_t unit = w / a.splits;
+  k.split = w - unit * a.splits;
+  k.lp = unit / per;
+  k.t += static_cast<uint32_t>(k.trials) * static_cast<uint32_t>(unit - k.lp * per);
+  return k;
+}
+
+// Work of one lane of lane group w: decode, prepare, sample, sum; the sums of
+// its trials in s1, s2 (zero beyond them).  rk0/rk1 are the ten Philox round
+// keys (parameter space in the single-scan kernel, registers in the batched
+// one); fx the fixed-point functors' table.
 template <int N, class F, int PREC>
-__device__ __forceinline__ void unit_split_lane(const ScanArgs& a, const uint32_t* rk0,
-                                                const uint32_t* rk1, const void* table,
-                                                const float* dimc, const int64_t* fx,
-                                                int64_t us, int lane, double& s1,
-                                                double& s2) {
-  const int64_t unit = us / a.splits;
-  const int64_t split = us - unit * a.splits;
-  const int64_t lp = unit / a.T;
-  const uint32_t t = static_cast<uint32_t>(unit - lp * a.T);
-  const int64_t p = a.first + lp;
-  if (!ZMC_CHECK(a.dbg, us >= 0 && lp < a.count && split < a.splits, kDbgGridIndex, us))
+__device__ __forceinline__ void lane_sums(const ScanArgs& a, const uint32_t* rk0,
+                                          const uint32_t* rk1, const void* table,
+                                          const float* dimc, const int64_t* fx,
+                                          const LaneWork& k, int lane, double* s1, double* s2) {
+  const int64_t p = a.first + k.lp;
+  if (!ZMC_CHECK(a.dbg, k.lp >= 0 && k.lp < a.count && k.split < a.splits &&
+                            k.t + k.trials <= static_cast<uint32_t>(a.T),
+                 kDbgGridIndex, k.lp))
     return;
 
   F f{};
   load_params<N>(a, table, dimc, p, f);
   if constexpr (FxOf<F, PREC>::kTable != kFxNone) {
     if (!f.ok) {
-      sample_unit_wide<N, typename FxOf<F, PREC>::Wide, PREC>(a, table, p, t, split, lane, s1,
-                                                              s2);
+      sample_unit_wide<N, typename FxOf<F, PREC>::Wide, PREC>(a, table, p, k.t, k.split, lane,
+                                                              s1, s2);
       return;
     }
     f.fx = fx;
   }
-  typename FxOf<F, PREC>::Acc acc;
-  sample_unit<N, F, PREC>(a, rk0, rk1, f, p, t, split, lane, acc);
-  s1 = acc.sum1();
-  s2 = acc.sum2();
+  if constexpr (max_trials<F, PREC>() > 1) {
+    if (k.trials == 4) {
+      sample_trials<N, F, PREC, 4>(a, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
+      return;
+    }
+    if (k.trials == 2) {
+      sample_trials<N, F, PREC, 2>(a, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
+      return;
+    }
+  }
+  sample_trials<N, F, PREC, 1>(a, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
 }
 
-// Reduce (s1, s2) over the `lanes` threads of each unit-split, in a fixed
-// order.  Every thread of the block must call it.  Lane 0 of the unit-split
-// returns the totals.
-__device__ __forceinline__ void reduce_unit_split(const ScanArgs& a, double& s1,
-                                                  double& s2, double* red) {
+// Cross-warp sums of a block: 16 warps of up to 2 kMaxLaneTrials values.
+constexpr int kReduceDoubles = 16 * 2 * kMaxLaneTrials;
+
+// Reduce V values per thread (a power of two) over the `lanes` threads of each
+// lane group, in a fixed order.  Within a warp: a butterfly in which, at each of
+// the first steps, the two partners each keep half of the values they still hold
+// and send the other half, so that V values cost V - 1 FP64 adds and one more
+// per further step instead of V per step (an FP64 add holds the SM's one FP64
+// unit for 16 clocks a warp; for four trials in 32 lanes 9 adds instead of 40).
+// Every value's sum is the same tree of the same numbers either way.  Wider lane
+// groups then add the warps' sums from shared memory, in order.  Every thread of
+// the block calls it; afterwards the threads of a lane group's first warp hold
+// its sums, this one values owner[0] .. owner[0] + owner[1] - 1 in x[0 ..).
+template <int V>
+__device__ __forceinline__ void reduce_lanes(const ScanArgs& a, double (&x)[V], double* red,
+                                             int* owner) {
   const int width = a.lanes < 32 ? a.lanes : 32;
-  for (int m = width >> 1; m >= 1; m >>= 1) {
-    s1 += __shfl_xor_sync(0xffffffffu, s1, m);
-    s2 += __shfl_xor_sync(0xffffffffu, s2, m);
+  const int lane = threadIdx.x & 31;
+  int held = V;   // values this thread still holds, in x[0 .. held)
+  int first = 0;  // the first of them
+  int m = width >> 1;
+#pragma unroll
+  for (int h = V >> 1; h >= 1; h >>= 1) {
+    if (m < 1) break;
+    const bool up = (lane & m) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double mine = up ? x[i + h] : x[i];
+      const double other = up ? x[i] : x[i + h];
+      x[i] = mine + __shfl_xor_sync(0xffffffffu, other, m);
+    }
+    if (up) first += h;
+    held = h;
+    m >>= 1;
   }
+  for (; m >= 1; m >>= 1)  // one value left (held == 1)
+    x[0] += __shfl_xor_sync(0xffffffffu, x[0], m);
+  owner[0] = first;
+  owner[1] = held;
   if (a.lanes > 32) {
+    // x[0] is value `first` of this warp (held == 1: 32 lanes >= V)
     const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) {
-      red[2 * warp] = s1;
-      red[2 * warp + 1] = s2;
-    }
+    if ((lane & (32 / V - 1)) == 0) red[warp * V + first] = x[0];
     __syncthreads();
-    if ((threadIdx.x & (a.lanes - 1)) == 0) {
-      const int wpu = a.lanes >> 5;
-      double t1 = red[2 * warp], t2 = red[2 * warp + 1];
-      for (int w = 1; w < wpu; ++w) {
-        t1 += red[2 * (warp + w)];
-        t2 += red[2 * (warp + w) + 1];
-      }
-      s1 = t1;
-      s2 = t2;
+    const int wpu = a.lanes >> 5;
+    if ((warp & (wpu - 1)) == 0) {
+      double t = red[warp * V + first];
+      for (int w = 1; w < wpu; ++w) t += red[(warp + w) * V + first];
+      x[0] = t;
     }
   }
+}
+
+// Reduce a block's lane sums (sum g of V / 2 trials, then sum g^2) and write the
+// lane groups' partial sums, each from one thread.
+template <int V>
+__device__ __forceinline__ void write_sums(const ScanArgs& a, const LaneWork& k, bool active,
+                                           int lane, double (&x)[V], double* red) {
+  int owner[2];
+  reduce_lanes<V>(a, x, red, owner);
+  const int width = a.lanes < 32 ? a.lanes : 32;
+  const int copies = width * owner[1] / V;  // threads that hold the same values
+  if (active && lane < width && (copies <= 1 || (lane & (copies - 1)) == 0)) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+      if (i >= owner[1]) break;
+      const int v = owner[0] + i, u = v & (V / 2 - 1);
+      if (u >= k.trials) continue;
+      const int64_t us = (k.lp * a.T + k.t + u) * a.splits + k.split;
+      if (ZMC_CHECK(a.dbg, us >= 0 && us < a.n_us, kDbgPartialSlot, us))
+        a.partial[2 * us + (v >= V / 2 ? 1 : 0)] = x[i];
+    }
+  }
+}
+
+// A block's lane groups first_w .. first_w + units - 1 (units <= blockDim.x /
+// lanes): sample, reduce and write each trial's partial sums.  Every thread of
+// the block calls it.
+template <int N, class F, int PREC>
+__device__ __forceinline__ void block_work(const ScanArgs& a, const uint32_t* rk0,
+                                           const uint32_t* rk1, const void* table,
+                                           const float* dimc, const int64_t* fx,
+                                           int64_t first_w, int units, double* red) {
+  constexpr int kB = max_trials<F, PREC>();
+  const int lane = threadIdx.x & (a.lanes - 1);
+  const int local = threadIdx.x >> a.lanes_log2;
+  const bool active = local < units;
+  LaneWork k{0, 0, 0, 0};
+  double x[2 * kB];  // sum g of the trials, then sum g^2
+#pragma unroll
+  for (int u = 0; u < 2 * kB; ++u) x[u] = 0.0;
+  if (active) {
+    k = lane_work<kB>(a, first_w + local);
+    lane_sums<N, F, PREC>(a, rk0, rk1, table, dimc, fx, k, lane, x, x + kB);
+  }
+  if constexpr (kB > 1) {
+    // lane groups of one size lie together, the larger ones first
+    if (lane_trials(a, first_w) > 1) {
+      write_sums<2 * kB>(a, k, active, lane, x, red);
+      return;
+    }
+  }
+  double y[2] = {x[0], x[kB]};
+  write_sums<2>(a, k, active, lane, y, red);
 }
 
 template <int N, class F, int PREC>
 __global__ void __launch_bounds__(ZMC_LB_THREADS, ZMC_LB_MIN_BLOCKS)
 scan_kernel(const __grid_constant__ ScanArgs a) {
   extern __shared__ double smem[];
-  __shared__ double red[64];
+  __shared__ double red[kReduceDoubles];
   __shared__ float dimc[3 * ZMC_MAX_N];
   const int64_t* fx = nullptr;
   if constexpr (FxOf<F, PREC>::kTable != kFxNone) {
@@ -535,17 +697,11 @@ scan_kernel(const __grid_constant__ ScanArgs a) {
     fx = fx_table;
   }
   const void* table = stage_lists<N, F>(a, smem, dimc);
-  const int lane = threadIdx.x & (a.lanes - 1);
-  const int64_t us = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> a.lanes_log2) +
-                     (threadIdx.x >> a.lanes_log2);
-  double s1 = 0.0, s2 = 0.0;
-  if (us < a.n_us)
-    unit_split_lane<N, F, PREC>(a, a.rk0, a.rk1, table, dimc, fx, us, lane, s1, s2);
-  reduce_unit_split(a, s1, s2, red);
-  if (lane == 0 && us < a.n_us && ZMC_CHECK(a.dbg, us >= 0, kDbgPartialSlot, us)) {
-    a.partial[2 * us] = s1;
-    a.partial[2 * us + 1] = s2;
-  }
+  const int per_block = blockDim.x >> a.lanes_log2;
+  const int64_t first_w = static_cast<int64_t>(blockIdx.x) * per_block;
+  const int64_t left = a.n_lw - first_w;
+  block_work<N, F, PREC>(a, a.rk0, a.rk1, table, dimc, fx, first_w,
+                         left < per_block ? static_cast<int>(left) : per_block, red);
 }
 
 #ifndef __CUDACC_RTC__

@@ -42,7 +42,6 @@
 
 namespace zmc {
 
-TilePlan plan_batch_scan(const zmc_scan_desc* d);
 constexpr int kServeBlock = 256;
 
 using Clock = std::chrono::steady_clock;
@@ -102,6 +101,7 @@ struct zmc_server {
   zmc_server_opts opts{};
   size_t budget = 0;
   int device = 0;
+  int sm_count = 1;
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
   std::deque<std::shared_ptr<zmc::Request>> queue;
@@ -188,12 +188,19 @@ static void start_chunk(Request* r, int64_t c) {
   r->chunk_count = std::min(r->chunk_points, r->d.first_index + r->count - r->chunk_first);
   r->chunk_units = r->chunk_count * r->d.trials * r->tp.splits;
   const int64_t per_block = kServeBlock / r->tp.lanes;
-  r->chunk_tiles = (r->chunk_units + per_block - 1) / per_block;
   r->next_tile = 0;
   zmc_scan_desc dc = r->d;
   dc.first_index = r->chunk_first;
   dc.count = r->chunk_count;
   fill_scan_args(&dc, r->chunk_count, r->tp, r->d_vals, r->d_part, &r->args);
+  r->chunk_tiles = (r->args.n_lw + per_block - 1) / per_block;
+}
+
+// Evaluations of one tile of r's current chunk.
+static double tile_evals_of(const Request* r) {
+  const int64_t groups = (r->args.ngroups + r->tp.splits - 1) / r->tp.splits;
+  return static_cast<double>(r->chunk_units) / r->chunk_tiles * groups *
+         group_samples(r->d.N);
 }
 
 // Admission: device memory for lists, one chunk of partials, output buffers.
@@ -422,10 +429,7 @@ static void run_loop(zmc_server* s) {
       double left = budget;
       for (size_t i = 0; i < ready.size() && tiles_used < s->tile_cap; ++i) {
         Request* r = ready[i].get();
-        const int G = group_samples(r->d.N);
-        const int64_t per_block = kServeBlock / r->tp.lanes;
-        const int64_t groups = (r->args.ngroups + r->tp.splits - 1) / r->tp.splits;
-        const double tile_evals = static_cast<double>(per_block) * groups * G;
+        const double tile_evals = tile_evals_of(r);
         const double allot = (i == 0 && ready.size() > 1) ? std::max(budget * 0.25, tile_evals)
                                                          : left;
         if (i > 0 && left < tile_evals) break;
@@ -474,8 +478,8 @@ static void run_loop(zmc_server* s) {
           for (int64_t t = picks[i].tile_begin; t < picks[i].tile_end; ++t) {
             BatchTile bt;
             bt.scan = i;
-            bt.first_us = t * per_block;
-            bt.units = static_cast<int32_t>(std::min(per_block, r->chunk_units - bt.first_us));
+            bt.first_w = t * per_block;
+            bt.units = static_cast<int32_t>(std::min(per_block, r->args.n_lw - bt.first_w));
             h_tiles[nt++] = bt;
           }
           if (r->args.stage_smem)
@@ -486,11 +490,8 @@ static void run_loop(zmc_server* s) {
       for (int i = 0; i < nsc; ++i) {
         Request* r = picks[i].r.get();
         h_args[i] = r->args;
-        const int G = group_samples(r->d.N);
-        const int64_t per_block = kServeBlock / r->tp.lanes;
-        const int64_t groups = (r->args.ngroups + r->tp.splits - 1) / r->tp.splits;
         st.evals += static_cast<double>(picks[i].tile_end - picks[i].tile_begin) *
-                    per_block * groups * G;
+                    tile_evals_of(r);
         if (picks[i].completes_chunk) {
           const int buf = static_cast<int>(r->chunk % 2);
           FinalizeArgs f;
@@ -641,6 +642,8 @@ int zmc_server_create(size_t mem_budget_bytes, const zmc_server_opts* opts, zmc_
   s->opts = o;
   s->budget = mem_budget_bytes;
   cudaError_t e = cudaGetDevice(&s->device);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, s->device);
   s->tile_cap = int64_t(1) << 20;
   s->stage_bytes = s256(sizeof(ScanArgs) * o.max_active) + s256(sizeof(BatchTile) * s->tile_cap) +
                    s256(sizeof(FinalizeArgs) * o.max_active) +
