@@ -42,11 +42,12 @@ int batch_blocks_per_sm(int precision, int block, size_t smem, int* out) {
 }
 
 constexpr int kBatchBlock = 256;
-// Sample groups per lane that bound one tile's work (tiles stay
+// Sample groups per lane (over its trials) that bound one tile's work (tiles stay
 // short next to the whole batch, so the longest-first order balances the SMs).
 constexpr int64_t kBatchGroupsPerLane = 1024;
 // Lanes per unit-split: the largest power of two <= 32 leaving each lane at
-// least this many sample groups (plain FP32 lane sums: 64).  Long lanes spend less of their time in the FP64
+// least this many sample groups, over all the trials it samples (plain FP32 lane
+// sums: 64 of each trial).  Long lanes spend less of their time in the FP64
 // epilogue on GB300's narrow FP64 unit: measured, 512 against 64 makes the 2048
 // small scans of the serving mix 6 % faster in one launch and leaves the uneven
 // 256-scan batch unchanged.
@@ -54,11 +55,20 @@ constexpr int64_t kBatchGroupsPerLane = 1024;
 #define ZMC_BATCH_LANE_GROUPS 512
 #endif
 
-TilePlan plan_batch_scan(const zmc_scan_desc* d) {
+int64_t scan_calls(const zmc_scan_desc* d, int64_t count) {
+  const int G = group_samples(d->N);
+  return count * d->trials * ((d->samples_per_point + G - 1) / G) * group_calls(d->N);
+}
+
+TilePlan plan_batch_scan(const zmc_scan_desc* d, int trials, int64_t lane_calls,
+                         int64_t least_groups) {
   TilePlan tp;
   const int G = group_samples(d->N);
   const int64_t Q = (d->samples_per_point + G - 1) / G;
   tp.block = kBatchBlock;
+  // Lanes that take several trials take fewer sample groups of each instead, so
+  // that the tiles stay as short.
+  tp.trials = std::min(trials, max_lane_trials(d));
   int tl = 0, tb = 0, tg = 0;
   if (!d->tile_lanes && !d->tile_splits &&
       tune_find(d->precision, d->integrand_id, d->N, d->samples_per_point, &tl, &tb, &tg)) {
@@ -68,16 +78,23 @@ TilePlan plan_batch_scan(const zmc_scan_desc* d) {
     tp.splits = static_cast<int>(std::min<int64_t>(std::max<int64_t>(1, (Q + per - 1) / per), Q));
     return tp;
   }
+  // Sample groups of each trial per lane, at most.
+  const int64_t groups =
+      std::min(kBatchGroupsPerLane / tp.trials,
+               std::max(least_groups, lane_calls / (group_calls(d->N) * tp.trials)));
   int lanes = d->tile_lanes;
   if (!lanes) {
-    const int64_t min_groups = d->precision == ZMC_FP32 ? 64 : ZMC_BATCH_LANE_GROUPS;
+    const int64_t min_groups =
+        d->precision == ZMC_FP32
+            ? std::min<int64_t>(64, groups)
+            : std::min<int64_t>(ZMC_BATCH_LANE_GROUPS / tp.trials, groups);
     lanes = 32;
     while (lanes > 1 && Q / lanes < min_groups) lanes >>= 1;
   }
   tp.lanes = std::min(lanes, kBatchBlock);
   int64_t splits = d->tile_splits;
   if (!splits) {
-    const int64_t per = int64_t(tp.lanes) * kBatchGroupsPerLane;
+    const int64_t per = int64_t(tp.lanes) * groups;
     splits = std::max<int64_t>(1, (Q + per - 1) / per);
   }
   tp.splits = static_cast<int>(std::min<int64_t>(std::max<int64_t>(splits, 1), Q));
@@ -194,7 +211,20 @@ int batch_create(const zmc_scan_desc* d, zmc_scan_out* o, int n, int flags, zmc_
   int dev = 0, sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
-  for (int i = 0; i < n; ++i) plans[i] = plan_batch_scan(&d[i]);
+  // Philox calls per lane that give each precision's launch kBatchWaves lanes per
+  // resident thread (two 256-thread blocks per SM), and trials per lane: as many
+  // as leave the launch kBatchRounds tiles per SM.
+  int64_t lane_calls[3] = {0, 0, 0};
+  for (int i = 0; i < n; ++i) lane_calls[d[i].precision] += scan_calls(&d[i], counts[i]);
+  for (auto& c : lane_calls) c /= kBatchWaves * 2 * kBatchBlock * std::max(sm, 1);
+  for (int b = kMaxLaneTrials; b >= 1; b >>= 1) {
+    int64_t tiles = 0;
+    for (int i = 0; i < n; ++i) {
+      plans[i] = plan_batch_scan(&d[i], b, lane_calls[d[i].precision], kBatchLeastGroups);
+      tiles += batch_tiles(&d[i], counts[i], plans[i]);
+    }
+    if (tiles >= kBatchRounds * std::max(sm, 1)) break;
+  }
 
   zmc_batch* b = new (std::nothrow) zmc_batch();
   if (!b) return fail(ZMC_ENOMEM, "host allocation failed");

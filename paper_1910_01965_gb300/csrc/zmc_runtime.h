@@ -56,9 +56,26 @@ ScanLayout layout_for(const zmc_scan_desc* d, int64_t count, const TilePlan& tp)
 int64_t chunk_points_for(const zmc_scan_desc* d, int64_t count, const TilePlan& tp);
 // The most trials of a point that one lane of this scan's kernel samples.
 int max_lane_trials(const zmc_scan_desc* d);
-// The plan of a batched or served scan, and the number of tiles of `count` points.
-TilePlan plan_batch_scan(const zmc_scan_desc* d);
+// Philox calls of a scan of `count` points.
+int64_t scan_calls(const zmc_scan_desc* d, int64_t count);
+// The plan of a batched or served scan with at most `trials` trials per lane and
+// about `lane_calls` Philox calls per lane, but no lane shorter than
+// `least_groups` sample groups; and the number of tiles of `count` points.
+TilePlan plan_batch_scan(const zmc_scan_desc* d, int trials, int64_t lane_calls,
+                         int64_t least_groups);
 int64_t batch_tiles(const zmc_scan_desc* d, int64_t count, const TilePlan& tp);
+// A persistent launch gets this many lanes per resident thread, if they keep
+// kBatchLeastGroups sample groups each.  Measured on GB300 on small batches: 27
+// scans (4.2e7 evaluations) 640 us with lanes of up to 1024 groups whatever the
+// batch's size, 150 / 143 / 144 us with 1 / 2 / 4; 37 scans (1.3e8) 1314 us and
+// 502 / 460 / 456 us.  Lanes of at least 32 groups against 64: 87 and 125 us for
+// 29 scans of 1.3e7 evaluations; 16 gives no more.
+constexpr int64_t kBatchWaves = 4;
+constexpr int64_t kBatchLeastGroups = 32;
+// Tiles per SM from which on lanes take several trials in the persistent kernel:
+// a launch with fewer is short of independent work (4.2e7 evaluations with four
+// trials per lane 1019 us, one 640 us; 5.4e9 in 6454 tiles 12.68 and 12.98 ms).
+constexpr int64_t kBatchRounds = 12;
 // Lane groups of a launch over `count` points (and how many of them take four
 // and two trials, may be null).
 int64_t lane_groups_of(const zmc_scan_desc* d, int64_t count, const TilePlan& tp, int64_t* lu4,

@@ -43,3 +43,37 @@ def test_trials_do_not_depend_on_their_company(zmc, prec, N, tiles):
             base = res
         assert np.array_equal(res["s1"], base["s1"][:, :T]), T
         assert np.array_equal(res["s2"], base["s2"][:, :T]), T
+
+
+@pytest.mark.parametrize("points,S,scans", [(1, 1, 1), (3, 1003, 5), (700, 4001, 3),
+                                            (6000, 3001, 40)])
+def test_batches_of_all_sizes_equal_solo_runs(zmc, points, S, scans):
+    """From a few lanes (short lanes, one trial each) to many rounds of tiles (lanes of
+    four trials): each scan of a batch equals its solo run with the batch's tiles."""
+    import torch
+    r = np.random.default_rng(scans)
+    descs, outs, keep, want = [], [], [], []
+    for i in range(scans):
+        N, T, prec = 1 + i % 8, (4, 5, 7, 1, 2)[i % 5], (2, 1, 0)[i % 3]
+        lens = [points] + [1] * (N - 1)
+        vals = r.uniform(0.2, 1.5, points + N - 1)
+        args = (GIDS[i % 6], N, [0.0] * N, [1.0] * N, lens, vals, S, T, 5 + i)
+        v = torch.from_numpy(vals).cuda()
+        d, k = zmc.make_desc(*args[:5], v, S, T, 5 + i, prec, zmc.ZMC_MEM_DEVICE)
+        res = [torch.empty(points, dtype=torch.float64, device="cuda") for _ in range(2)] + \
+            [torch.empty((points, T), dtype=torch.float64, device="cuda") for _ in range(2)]
+        o = zmc.zmc_scan_out()
+        o.mean, o.err, o.s1, o.s2 = (zmc._ptr(x) for x in res)
+        descs.append(d)
+        outs.append(o)
+        keep.append((v, k, res))
+        want.append((args, prec))
+    h = zmc.zmc_batch_create(descs, outs)
+    zmc.zmc_batch_run(h)
+    torch.cuda.synchronize()
+    for (args, prec), o, (_, _, res) in zip(want, outs, keep):
+        solo, _ = zmc.scan(*args, precision=prec, want_sums=True,
+                           tiles=(o.tile_lanes, o.tile_splits, o.tile_block))
+        assert np.array_equal(solo["s1"], res[2].cpu().numpy())
+        assert np.array_equal(solo["s2"], res[3].cpu().numpy())
+    zmc.zmc_batch_destroy(h)
