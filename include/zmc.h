@@ -63,7 +63,8 @@ typedef enum {
  * width, or an integrand that cancels strongly, keeps only FP32's 24 bits;
  * ZMC_FP64 has no such limit.  Per sample the FP32 error is ~1e-7 of g. */
 typedef enum {
-  ZMC_FP64 = 0,        /* FP64 samples, integrand and sums                 */
+  ZMC_FP64 = 0,        /* FP64 samples, integrand and sums (or 64-bit fixed
+                          point of at least that accuracy)                 */
   ZMC_FP32 = 1,        /* FP32 samples and integrand, plain FP32 lane sums  */
   ZMC_FP32_KAHAN = 2   /* FP32 samples and integrand, Kahan FP32 lane sums  */
 } zmc_precision;       /* cross-lane reduction and the statistics: FP64    */
@@ -120,7 +121,10 @@ enum {
  *                       0 = chosen by the planner/autotuner; otherwise
  *                       lanes per unit-split (power of two <= tile_block),
  *                       sample splits per (point, trial) unit, and threads
- *                       per block (64..512, multiple of 32)
+ *                       per block (64..512, multiple of 32).  Lanes and
+ *                       splits fix the order of a unit's sums; the block
+ *                       does not (left at 0, the launch may use blocks
+ *                       smaller than the one it reports)
  *  flags                ZMC_F_* bits
  *  chunk_points         zmc_scan_ex cuts the slice into chunks of this many
  *                       consecutive grid points (the batches of Sec. 2);

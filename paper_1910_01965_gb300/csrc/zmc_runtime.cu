@@ -271,37 +271,59 @@ int max_lane_trials(const zmc_scan_desc* d) {
   return d->trials >= 4 ? 4 : d->trials >= 2 ? 2 : 1;
 }
 
-// Trials per lane: 4, 2 or 1, whichever ends first by this model.  Blocks are
-// spread over the SMs in rounds (one 256-thread block keeps an SM busy), those
-// with more trials first; a block of 4 (2) trials takes 3.74 (1.92) times as long
-// as one of a single trial, having shared part of its Philox calls.  Measured on
-// the Gaussian at N = 4 (T = 4, 2^14 samples, 32 lanes): one round of blocks
-// takes 46 us with one trial and 165-172 us with four, so 1000 points (125
-// blocks of four trials on 152 SMs) run in 185 against 189 us, 1500 points (187
-// blocks, two rounds) in 345 against 235 us, 10^5 points in 13.5 against 14.2 ms.
-static int plan_lane_trials(const zmc_scan_desc* d, int64_t count, const TilePlan& tp, int sm) {
-  int best = 1;
-  double best_cost = 0.0;
+// The launch shape.  Blocks of 128 threads: one warp per SM sub-partition, so that
+// a short launch reaches all SMs and wastes less of its last turn; 256 where every
+// block stages a long list.  Measured on GB300 against 256-thread blocks: Gaussian
+// N = 4, T = 4, 2^14 samples, 10 points 53 -> 36 us, 700 points 144 -> 126 us;
+// with lists of 3000 values 464 -> 480 us.
+//
+// Trials per lane: the number whose launch ends first by this model.  A block of
+// 4 (2) trials takes 3.7 (1.9) times as long as one of a single trial, having
+// shared part of its Philox calls; blocks go to the SMs in turns, those with more
+// trials first.  On the same scan, 128-thread blocks of 1, 2, 4 trials: 700 points
+// 126, 138, 185 us; 1500 points 241, 230, 272 us; 40,000 points 5.78, 5.41,
+// 5.39 ms.  Over ten kernels and shapes the model's choice took 0.87 of the time
+// of 256-thread single-trial blocks (geometric mean), 2 % more than the best.
+constexpr int kLongLists = 1024;
+void plan_launch(const zmc_scan_desc* d, int64_t count, int sm, TilePlan* tp) {
+  static const double kCost[3] = {3.7, 1.9, 1.0};
+  int64_t nvals = 0;
+  for (int i = 0; i < d->M; ++i) nvals += d->list_len[i];
+  tp->launch_block = tp->block;
+  // the caller's and the tuner's blocks stay as they are
+  if (d->tile_block == 0 && tp->block == 256 && tp->lanes <= 128 &&
+      (nvals <= kLongLists || nvals > kMaxSmemVals))
+    tp->launch_block = 128;
+  const double per_block = static_cast<double>(tp->launch_block / tp->lanes);
+  double best = 0.0;
+  TilePlan t = *tp;
   sm = std::max(1, sm);
   for (int b = 1; b <= max_lane_trials(d); b <<= 1) {
-    TilePlan t = tp;
     t.trials = b;
     int64_t lu4 = 0, lu2 = 0;
     const int64_t lw = lane_groups_of(d, count, t, &lu4, &lu2);
-    const double per_block = static_cast<double>(tp.block / tp.lanes);
-    const double n4 = lu4 / per_block, n2 = lu2 / per_block, n1 = (lw - lu4 - lu2) / per_block;
-    const double first = n4 > 0 ? 3.74 : n2 > 0 ? 1.92 : 1.0;
-    const double rounds = std::ceil((n4 > 0 ? n4 : n2 > 0 ? n2 : n1) / sm) * first;
-    const double all = (3.74 * n4 + 1.92 * n2 + n1) / sm;
-    const double cost = n1 > 0 && first > 1.0 ? std::max(rounds, all + 0.5)
-                        : n2 > 0 && n4 > 0    ? std::max(rounds, all + 1.0)
-                                              : rounds;
-    if (b == 1 || cost < best_cost) {
-      best = b;
-      best_cost = cost;
+    const int64_t n[3] = {lu4, lu2, lw - lu4 - lu2};
+    // turns of the largest blocks; or all the work and half a block of the last
+    double first = 0.0, turns = 0.0, all = 0.0, last = 0.0;
+    for (int i = 0; i < 3; ++i) {
+      if (n[i] <= 0) continue;
+      const double blocks = n[i] / per_block / sm;
+      all += blocks * kCost[i];
+      last = kCost[i];
+      if (first == 0.0) {
+        first = kCost[i];
+        turns = std::ceil(blocks) * first;
+      }
+    }
+    double cost = last < first ? std::max(turns, all + 0.5 * last) : turns;
+    // a warp alone on its sub-partition takes 1.5 times as long
+    if (tp->launch_block <= 128) cost = std::max(cost, 1.5 * first);
+    cost += 0.2 * first;
+    if (b == 1 || cost < best) {
+      best = cost;
+      tp->trials = b;
     }
   }
-  return best;
 }
 
 static size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
@@ -381,7 +403,7 @@ static TilePlan plan_sums(const zmc_scan_desc* d, int64_t count, int sm, int tps
 
 TilePlan plan_with(const zmc_scan_desc* d, int64_t count, int sm, int tps) {
   TilePlan tp = plan_sums(d, count, sm, tps);
-  tp.trials = plan_lane_trials(d, count, tp, sm);
+  plan_launch(d, count, sm, &tp);
   return tp;
 }
 
@@ -469,19 +491,19 @@ int launch_scan_args(const zmc_scan_desc* d, const ScanArgs& a, const TilePlan& 
                      cudaStream_t stream) {
   if (a.n_us == 0) return ZMC_OK;
   if (is_user_integrand(d->integrand_id)) {
-    const int64_t per_block = tp.block / tp.lanes;
+    const int64_t per_block = tp.launch_block / tp.lanes;
     const int64_t grid = (a.n_lw + per_block - 1) / per_block;
     if (grid > 0x7fffffffLL) return fail(ZMC_EINVAL, "launch grid too large (%lld)", (long long)grid);
     const size_t smem = a.stage_smem ? static_cast<size_t>(a.nvals) * sizeof(double) : 0;
-    return user_launch(d, a, tp.block, grid, smem, stream);
+    return user_launch(d, a, tp.launch_block, grid, smem, stream);
   }
   ScanLaunchFn fn = scan_launcher(d->precision, d->integrand_id, d->N);
   if (!fn) return fail(ZMC_ENOTFOUND, "no kernel for integrand %d, N %d", d->integrand_id, d->N);
-  const int64_t per_block = tp.block / tp.lanes;
+  const int64_t per_block = tp.launch_block / tp.lanes;
   const int64_t grid = (a.n_lw + per_block - 1) / per_block;
   if (grid > 0x7fffffffLL) return fail(ZMC_EINVAL, "launch grid too large (%lld)", (long long)grid);
   const size_t smem = a.stage_smem ? static_cast<size_t>(a.nvals) * sizeof(double) : 0;
-  int e = fn(a, tp.block, grid, smem, stream);
+  int e = fn(a, tp.launch_block, grid, smem, stream);
   if (e != 0) return cuda_fail(static_cast<cudaError_t>(e), "sampling kernel launch");
   return ZMC_OK;
 }
@@ -759,10 +781,12 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
     zmc_scan_desc dc = *d;
     dc.first_index = d->first_index + k * cp;
     dc.count = n;
+    TilePlan tk = tp;  // the sums of the whole call, launched to suit the chunk
+    if (nch > 1) plan_launch(d, n, ds->prop.multiProcessorCount, &tk);
     ScanArgs a;
-    fill_scan_args(&dc, n, tp, vals_dev, reinterpret_cast<double*>(ws + L.partial), &a);
+    fill_scan_args(&dc, n, tk, vals_dev, reinterpret_cast<double*>(ws + L.partial), &a);
     ev.record(2 + 3 * k, stream);
-    rc = launch_scan_args(d, a, tp, stream);
+    rc = launch_scan_args(d, a, tk, stream);
     if (rc != ZMC_OK) {
       release();
       return rc;

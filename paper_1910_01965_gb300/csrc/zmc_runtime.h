@@ -14,7 +14,9 @@ struct TilePlan {
   int lanes = 32;   // threads summing one unit-split (power of two)
   int splits = 1;   // sample ranges per (point, trial) unit
   int block = 256;  // threads per block
-  int trials = 1;   // trials of a point that the same lanes sample (1, 2, 4)
+  // How the launch is shaped; neither changes a result.
+  int trials = 1;          // trials of a point that the same lanes sample (1, 2, 4)
+  int launch_block = 256;  // threads per block of the launch, at most `block`
 };
 
 // Byte offsets of each region inside one scan's device scratch.  The slice
@@ -40,6 +42,9 @@ TilePlan plan_tiles(int N, int64_t S, int T, int64_t count, int sm_count, int th
 // an autotuner entry for the scan's class when the caller leaves the tiles
 // open and one is recorded (memory reads only), else plan_tiles.
 TilePlan plan_with(const zmc_scan_desc* d, int64_t count, int sm, int tps);
+// The launch shape (trials, launch_block) of a launch over `count` points with the
+// sums of `tp`.
+void plan_launch(const zmc_scan_desc* d, int64_t count, int sm, TilePlan* tp);
 // plan_with for the current device (its properties from the device state),
 // after loading the autotuner's cache file once.
 int plan_for(const zmc_scan_desc* d, int64_t count, TilePlan* tp);
