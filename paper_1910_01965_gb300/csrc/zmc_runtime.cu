@@ -560,9 +560,9 @@ static bool is_pinned_host(const void* p, size_t bytes) {
   return pinned(p) && pinned(static_cast<const char*>(p) + bytes - 1);
 }
 
-// Page-locked staging buffers for chunked scans into pageable host arrays,
-// kept for reuse across calls (a process-wide free list; each call holds its
-// buffer for its duration, so concurrent calls never share one).
+// Page-locked staging buffers for chunked scans into pageable host arrays and
+// for small calls, kept for reuse across calls (a process-wide free list; each
+// call holds its buffer for its duration, so concurrent calls never share one).
 struct PinnedBuf {
   char* p = nullptr;
   size_t bytes = 0;
@@ -601,6 +601,12 @@ static void pinned_give(PinnedBuf b) {
     g_pin_free.erase(it);
   }
 }
+
+// Lists and outputs of a call that goes through a pinned buffer of this size.
+constexpr size_t kSmallCallBytes = size_t(1) << 18;
+// Blocks up to which they read the lists from host memory themselves (about a
+// microsecond each, against the copy's start-up on the stream).
+constexpr int64_t kListReadBlocks = 2048;
 
 // One output array of a chunk: where the finalize kernel wrote it on the
 // device, where it goes on the host, and its length in doubles.
@@ -678,11 +684,24 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
              is_pinned_host(o->s2, pb_all * T);
   const size_t per_chunk_doubles =
       static_cast<size_t>(cp) * (2 + (o->errw ? 1 : 0) + (o->s1 ? T : 0) + (o->s2 ? T : 0));
+  // A small call with host buffers keeps the GPU's copy engine out: the lists go
+  // through a pinned buffer, from which the blocks read them if they are few, and
+  // the finalize kernel writes the results into it.  Two to three copies from and
+  // into pageable memory took 18 us of the README call's 112 us.
+  const size_t out_doubles = static_cast<size_t>(count) *
+                             (2 + (o->errw ? 1 : 0) + (o->s1 ? T : 0) + (o->s2 ? T : 0));
+  int64_t list_doubles = 0;
+  for (int i = 0; i < d->M; ++i) list_doubles += d->list_len[i];
+  const size_t small_bytes = (static_cast<size_t>(list_doubles) + out_doubles) * sizeof(double);
+  const bool small = host && nch == 1 && !(d->flags & ZMC_F_TIMINGS) &&
+                     small_bytes <= kSmallCallBytes;
   PinnedBuf stage;
+  bool stage_in_use = false;  // by work enqueued on the stream
   cudaEvent_t ready[2] = {nullptr, nullptr}, copied[2] = {nullptr, nullptr};
   bool copies_enqueued = false;
   auto release = [&]() {
     if (copies_enqueued) cudaStreamSynchronize(cs);
+    if (stage_in_use) cudaStreamSynchronize(stream);
     for (int b = 0; b < 2; ++b) {
       if (ready[b]) cudaEventDestroy(ready[b]);
       if (copied[b]) cudaEventDestroy(copied[b]);
@@ -705,6 +724,11 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
     }
   }
 
+  if (small && (rc = pinned_take(kSmallCallBytes, &stage)) != ZMC_OK) {
+    release();
+    return rc;
+  }
+
   // Events: 0 start, 1 lists copied, then per chunk (sampling start, sampling
   // end, finalize end), then one after the last copy.
   EventSet ev;
@@ -719,9 +743,16 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
   int64_t nvals = 0;
   for (int i = 0; i < d->M; ++i) nvals += d->list_len[i];
   ev.record(0, stream);
-  if (host) {
+  if (small) std::memcpy(stage.p, d->list_vals, nvals * sizeof(double));
+  const int64_t blocks =
+      lane_groups_of(d, count, tp, nullptr, nullptr) / (tp.launch_block / tp.lanes);
+  if (small && blocks <= kListReadBlocks) {
+    vals_dev = reinterpret_cast<const double*>(stage.p);
+  } else if (host) {
     double* v = reinterpret_cast<double*>(ws + L.vals);
-    cudaError_t e = cudaMemcpyAsync(v, d->list_vals, nvals * sizeof(double),
+    const void* src = small ? static_cast<const void*>(stage.p) : d->list_vals;
+    stage_in_use = small;
+    cudaError_t e = cudaMemcpyAsync(v, src, nvals * sizeof(double),
                                     cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) {
       release();
@@ -741,6 +772,17 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
       dev[2] = o->errw ? o->errw + off : nullptr;
       dev[3] = o->s1 ? o->s1 + off * T : nullptr;
       dev[4] = o->s2 ? o->s2 + off * T : nullptr;
+      return;
+    }
+    if (small) {
+      double* at = reinterpret_cast<double*>(stage.p) + nvals;
+      double* const want[5] = {o->mean, o->err, o->errw, o->s1, o->s2};
+      for (int i = 0; i < 5; ++i) {
+        const size_t len = static_cast<size_t>(n) * (i < 3 ? 1 : T);
+        dev[i] = want[i] ? at : nullptr;
+        cps[i] = {want[i], at, want[i] ? len : 0};
+        if (want[i]) at += len;
+      }
       return;
     }
     const size_t bo = static_cast<size_t>(b) * cp;
@@ -786,6 +828,7 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
     ScanArgs a;
     fill_scan_args(&dc, n, tk, vals_dev, reinterpret_cast<double*>(ws + L.partial), &a);
     ev.record(2 + 3 * k, stream);
+    stage_in_use = small;
     rc = launch_scan_args(d, a, tk, stream);
     if (rc != ZMC_OK) {
       release();
@@ -816,7 +859,7 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
     }
     o->launches += 2;
     ev.record(4 + 3 * k, stream);
-    if (!host) continue;
+    if (!host || small) continue;
     cudaStream_t cstream = piped ? cs : stream;
     if (piped) {
       cudaEventRecord(ready[b], stream);
@@ -864,9 +907,22 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
     copies_enqueued = false;  // ordered behind the stream: no wait on the copy stream
   }
   ev.record(ev_last, stream);
+  if (small) {
+    const cudaError_t e = cudaStreamSynchronize(stream);
+    stage_in_use = false;
+    if (e != cudaSuccess) {
+      release();
+      return cuda_fail(e, "cudaStreamSynchronize");
+    }
+    double* dev[5];
+    OutCopy cps[5];
+    chunk_outputs(0, count, 0, dev, cps);
+    for (auto& c : cps)
+      if (c.n) std::memcpy(c.dst, c.src, c.n * sizeof(double));
+  }
   release();
 
-  if (host || timed || ZMC_DEBUG || (d->flags & ZMC_F_SYNC)) {
+  if ((host && !small) || timed || ZMC_DEBUG || (d->flags & ZMC_F_SYNC)) {
     cudaError_t e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
   }

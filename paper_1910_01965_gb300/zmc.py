@@ -9,6 +9,7 @@ kernels.  The names mirror the C entry points (``zmc_scan``, ``zmc_scan_ex``,
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 import threading
 
@@ -178,11 +179,14 @@ SIGNATURES = [
 
 _lock = threading.Lock()
 _lib = None
+_scan_addr = None  # zmc_scan taking its arrays as plain addresses
 
 
 def load(path: str = LIBRARY):
     """Load libzmc.so (built by __graft_entry__.build()); raise if missing."""
-    global _lib
+    global _lib, _scan_addr
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -195,8 +199,16 @@ def load(path: str = LIBRARY):
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
+        _scan_addr = lib["zmc_scan"]  # a function object of its own
+        _scan_addr.restype = ctypes.c_int
+        _scan_addr.argtypes = [ctypes.c_void_p if a in (_dp, _i64p) else a
+                               for a in dict((n, a) for n, _, a in SIGNATURES)["zmc_scan"]]
         _lib = lib
         return lib
+
+
+def _addr(a: np.ndarray) -> int:
+    return a.__array_interface__["data"][0]
 
 
 def _check(rc: int):
@@ -255,13 +267,12 @@ def zmc_scan(gid, N, lo, hi, lengths, values, S, T, seed):
     hi = np.ascontiguousarray(hi, np.float64)
     L = np.ascontiguousarray(lengths, np.int64)
     v = np.ascontiguousarray(values, np.float64)
-    P = int(np.prod(L))
+    P = math.prod(L.tolist())
     mean = np.empty(P)
     err = np.empty(P)
-    _check(load().zmc_scan(int(gid), int(N), lo.ctypes.data_as(_dp), hi.ctypes.data_as(_dp),
-                           len(L), L.ctypes.data_as(_i64p), v.ctypes.data_as(_dp),
-                           int(S), int(T), int(seed), mean.ctypes.data_as(_dp),
-                           err.ctypes.data_as(_dp)))
+    load()
+    _check(_scan_addr(int(gid), int(N), _addr(lo), _addr(hi), len(L), _addr(L), _addr(v), int(S),
+                      int(T), int(seed), _addr(mean), _addr(err)))
     return mean, err
 
 
@@ -470,6 +481,12 @@ class _Keep:
         return a
 
 
+def _set_ptr(struct, field: str, address: int):
+    """Store an address in a pointer field (ctypes' own pointer objects cost
+    microseconds each)."""
+    ctypes.c_void_p.from_buffer(struct, getattr(type(struct), field).offset).value = address
+
+
 def make_desc(gid, N, lo, hi, lengths, values=None, S=1, T=1, seed=0,
               precision=ZMC_FP32_KAHAN, mem=ZMC_MEM_HOST, first_index=0, count=-1,
               stream=None, tiles=(0, 0, 0), flags=0, keep=None, chunk_points=0):
@@ -481,15 +498,16 @@ def make_desc(gid, N, lo, hi, lengths, values=None, S=1, T=1, seed=0,
     hi_a = keep.arr(hi, np.float64)
     L = keep.arr(lengths, np.int64)
     d.integrand_id, d.N, d.M = int(gid), int(N), len(L)
-    d.lo, d.hi = lo_a.ctypes.data_as(_dp), hi_a.ctypes.data_as(_dp)
-    d.list_len = L.ctypes.data_as(_i64p)
+    _set_ptr(d, "lo", _addr(lo_a))
+    _set_ptr(d, "hi", _addr(hi_a))
+    _set_ptr(d, "list_len", _addr(L))
     if mem == ZMC_MEM_HOST:
         v = keep.arr(values, np.float64)
-        d.list_vals = v.ctypes.data_as(_dp)
+        _set_ptr(d, "list_vals", _addr(v))
     else:
         ptr = values if isinstance(values, int) else values.data_ptr()
         keep.items.append(values)
-        d.list_vals = ctypes.cast(ctypes.c_void_p(ptr), _dp)
+        _set_ptr(d, "list_vals", ptr)
     d.samples_per_point, d.trials, d.seed = int(S), int(T), int(seed) & (2 ** 64 - 1)
     d.precision, d.mem = int(precision), int(mem)
     d.first_index, d.count = int(first_index), int(count)
@@ -516,7 +534,7 @@ def scan(gid, N, lo, hi, lengths, values, S, T, seed, precision=ZMC_FP32_KAHAN,
     d, keep = make_desc(gid, N, lo, hi, lengths, values, S, T, seed, precision,
                         ZMC_MEM_HOST, first_index, count, None, tiles, flags,
                         chunk_points=chunk_points)
-    P = int(np.prod(np.asarray(lengths, np.int64)))
+    P = math.prod(int(v) for v in lengths)
     n = (P - first_index) if count < 0 else count
     res = {"mean": np.empty(n), "err": np.empty(n)}
     if want_errw:
@@ -525,9 +543,8 @@ def scan(gid, N, lo, hi, lengths, values, S, T, seed, precision=ZMC_FP32_KAHAN,
         res["s1"] = np.empty((n, T))
         res["s2"] = np.empty((n, T))
     o = zmc_scan_out()
-    o.mean, o.err = _ptr(res["mean"]), _ptr(res["err"])
-    o.errw = _ptr(res.get("errw"))
-    o.s1, o.s2 = _ptr(res.get("s1")), _ptr(res.get("s2"))
+    for name, a in res.items():
+        _set_ptr(o, name, _addr(a))
     zmc_scan_ex(d, o)
     return res, o
 
