@@ -285,6 +285,99 @@ ZMC_FX double fx_exp2neg(uint64_t q, const int64_t* table) {
   return fx_bits_double((static_cast<uint64_t>(1023 - n - z) << 52) + (m >> 1));
 }
 
+// A biased product shifted up to the top of its range (62 bits), with its exponent,
+// so that a long product of small factors keeps its precision.
+ZMC_FX int64_t fx_normalise(int64_t g, int* exponent) {
+  const int64_t m = g - kFxBias;
+  const int32_t h = fx_top(m);
+  const int c = fx_clz(static_cast<uint32_t>(h ^ (h >> 31)));
+  const int z = c > 2 ? c - 2 : 0;
+  *exponent -= z;
+  return static_cast<int64_t>(static_cast<uint64_t>(m) << z) + kFxBias;
+}
+
+// The double nearest to g 2^(S - 62), |S| <= 900 (g of any sign, 0 included).
+ZMC_FX double fx_to_double(int64_t g, int S) {
+  const uint64_t sign = static_cast<uint64_t>(g) & (uint64_t(1) << 63);
+  uint64_t m = static_cast<uint64_t>(g < 0 ? -g : g);
+  const uint32_t h = static_cast<uint32_t>(m >> 32);
+  const int z = h ? fx_clz(h) : 32 + fx_clz(static_cast<uint32_t>(m));
+  if (z >= 64) return 0.0;
+  m = ((m << z) >> 10) + 1;  // bit 53 leads
+  return fx_bits_double(sign | ((static_cast<uint64_t>(1023 + S - z) << 52) + (m >> 1)));
+}
+
+// round(v 2^k) for |v 2^k| < 2^63.
+ZMC_FX int64_t fx_fix(double v, int k) {
+  const uint64_t u = fx_double_bits(v);
+  const int ex = static_cast<int>((u >> 52) & 0x7ff);
+  const uint64_t m = ex ? (u & 0xfffffffffffffull) | (uint64_t(1) << 52) : 0;
+  const int s = 1075 - ex - k;  // right shift of m
+  const uint64_t w = s <= 0 ? m << -s : s > 54 ? 0 : ((m >> (s - 1)) + 1) >> 1;
+  return u >> 63 ? -static_cast<int64_t>(w) : static_cast<int64_t>(w);
+}
+
+// (c u) >> 32 for a 64-bit c with signed low half (ch, cl) and a signed 32-bit u.
+ZMC_FX int64_t fx_mul32(int32_t ch, int32_t cl, int32_t u) {
+  return fx_wide(ch, u) + fx_mulhi(cl, u);
+}
+
+// Twofold numbers hi + lo for the polynomial's constants.
+struct FxTwo {
+  double hi, lo;
+};
+ZMC_FX FxTwo fx_two_sum(double a, double b) {
+  const double s = a + b, t = s - a;
+  return {s, (a - (s - t)) + (b - t)};
+}
+ZMC_FX FxTwo fx_two_mul(FxTwo a, double b) {
+  const double p = a.hi * b;
+  return {p, fma(a.hi, b, -p) + a.lo * b};
+}
+
+// 1 + x y^2, y = a + w (2 v + 1) 2^-24, as c0 + u (c1 + u c2) in the centred field
+// u = (v - 2^22) 2^-23, all over 2^s: 2^62 times, c0 and c1 with the bias.
+struct FxPoly {
+  int64_t c0, c1, c2;
+  int s;
+  bool ok;
+};
+ZMC_FX FxPoly fx_poly(double x, double a, double w) {
+  const double k = 0.5 + 0x1p-24;
+  const double wk = w * k;
+  FxTwo m = fx_two_sum(a, wk);
+  m.lo += fma(w, k, -wk);
+  const FxTwo mw = fx_two_mul(m, w);
+  FxTwo mm = fx_two_mul(m, m.hi);
+  mm.lo += m.hi * m.lo;
+  const FxTwo xmm = fx_two_mul(mm, x);
+  FxTwo c0 = fx_two_sum(1.0, xmm.hi);
+  c0.lo += xmm.lo;
+  const FxTwo c1 = fx_two_mul(mw, 2.0 * x);
+  const double ww = w * w;
+  const FxTwo c2 = fx_two_mul({ww, fma(w, w, -ww)}, x);
+  const double q0 = fabs(c0.hi), q1 = fabs(c1.hi), q2 = fabs(c2.hi);
+  double b = q0 + 0.5 * q1 + 0.25 * q2;
+  b = q1 + 0.5 * q2 > b ? q1 + 0.5 * q2 : b;
+  b = q2 > b ? q2 : b;
+  FxPoly r{0, 0, 0, 0, fx_below(b, 60) && fx_below(x, 200) && fx_below(a, 200) &&
+                           fx_below(w, 200)};
+  if (!r.ok) return r;
+  // b < 2^s with room for the roundings
+  r.s = static_cast<int>((fx_double_bits(b * (1.0 + 0x1p-20)) >> 52) & 0x7ff) - 1022;
+  r.c0 = fx_fix(c0.hi, 62 - r.s) + fx_fix(c0.lo, 62 - r.s) + kFxBias;
+  r.c1 = fx_fix(c1.hi, 62 - r.s) + fx_fix(c1.lo, 62 - r.s) + kFxBias;
+  r.c2 = fx_fix(c2.hi, 62 - r.s) + fx_fix(c2.lo, 62 - r.s) + kFxBias;
+  return r;
+}
+
+// Its value at field v, times 2^(62 - s), biased.
+ZMC_FX int64_t fx_poly_eval(int64_t c0, int64_t c1, int64_t c2, uint32_t v) {
+  const int32_t u = static_cast<int32_t>((v << 9) ^ 0x80000000u);  // u 2^32
+  const int64_t t = c1 + fx_mul32(fx_top(c2), fx_low(c2), u);
+  return c0 + fx_mul32(fx_top(t), fx_low(t), u);
+}
+
 // round(v K 2^(59 - 61)) for a constant K below 2^63 and |v K 2^-61| < 31.9
 // (from 16 on only a v > 0, whose result is read as unsigned).
 ZMC_FX int64_t fx_scale59(double v, uint64_t K) {

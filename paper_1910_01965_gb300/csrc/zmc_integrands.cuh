@@ -180,7 +180,7 @@ struct Gauss64Wide {
 };
 
 template <int N>
-struct Poly64 {
+struct Poly64Wide {
   static constexpr bool kPerDim = true;
   static constexpr bool kTable = false;
   static constexpr bool kUsesSamples = true;

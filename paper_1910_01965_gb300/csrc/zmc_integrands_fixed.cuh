@@ -224,6 +224,40 @@ struct Gauss64 {
   }
 };
 
+// prod_k (1 + x_k y_k^2), each factor over a power of two above its largest
+// value in the box, so that every product is at most 1; the powers return in g's
+// exponent.  In range: factors below 2^60.  The sums stay FP64.
+template <int N>
+struct Poly64 {
+  static constexpr bool kPerDim = true;
+  static constexpr bool kTable = false;
+  static constexpr bool kUsesSamples = true;
+  static constexpr int kCallsInFlight = 1;
+  static constexpr int kFixedM = 0;
+  using unit_t = uint32_t;
+  bool ok = true;
+  int scale = 0;
+  int64_t c0[N], c1[N], c2[N];
+  __device__ void set(int i, double xi, double ai, double bi) {
+    const FxPoly p = fx_poly(xi, ai, bi - ai);
+    ok = ok && p.ok;
+    scale += p.s;
+    c0[i] = p.c0;
+    c1[i] = p.c1;
+    c2[i] = p.c2;
+  }
+  __device__ double eval(const uint32_t* v) const {
+    int64_t g = fx_poly_eval(c0[0], c1[0], c2[0], v[0]);
+    int e = scale;
+#pragma unroll
+    for (int k = 1; k < N; ++k) {
+      if (k > 1 && k % 2 == 0) g = fx_normalise(g, &e);  // every second factor
+      g = fx_mul62(g, fx_poly_eval(c0[k], c1[k], c2[k], v[k]));
+    }
+    return fx_to_double(g - kFxBias, e);
+  }
+};
+
 __device__ __forceinline__ void fx_fill(int64_t* dst, const int64_t* src, int n) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
 }
@@ -233,6 +267,14 @@ __device__ __forceinline__ void fx_fill_tables(int64_t* dst) {
   fx_fill(dst, kFxTables.c, kFxCosEntries);
   fx_fill(dst + kFxCosEntries, kFxTables.e, kFxExpEntries);
 }
+
+template <int N>
+struct FxOf<Poly64<N>, kPrecFP64> {
+  static constexpr int kTable = kFxNoTable;
+  static constexpr size_t kStaticBytes = 0;
+  using Wide = Poly64Wide<N>;
+  using Acc = LaneAcc<kPrecFP64>;
+};
 
 template <class W>
 struct FxCosOf {

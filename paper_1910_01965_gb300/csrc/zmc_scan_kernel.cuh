@@ -37,8 +37,9 @@ enum { kPrecFP64 = ZMC_FP64, kPrecFP32 = ZMC_FP32, kPrecFP32K = ZMC_FP32_KAHAN }
 // ZMC_CALLS_IN_FLIGHT, when defined, overrides every functor's kCallsInFlight
 // (independent Philox calls per lane per loop block in the FP32 paths).
 
-// Fixed-point tables a functor reads from shared memory (0: none).
-enum { kFxNone = 0, kFxCosTable = 1, kFxExpTable = 2 };
+// How a functor evaluates: in floating point, or in fixed point with one of the
+// tables in shared memory or with none.
+enum { kFxNone = 0, kFxCosTable = 1, kFxExpTable = 2, kFxNoTable = 3 };
 
 // The fixed-point functors specialise this: their table, their lane sums and
 // the FP64 functor that takes the parameters outside their range.
@@ -562,7 +563,7 @@ __device__ __forceinline__ void lane_sums(const ScanArgs& a, const uint32_t* rk0
                                                               s1, s2);
       return;
     }
-    f.fx = fx;
+    if constexpr (FxOf<F, PREC>::kTable != kFxNoTable) f.fx = fx;
   }
   if constexpr (max_trials<F, PREC>() > 1) {
     if (k.trials == 4) {
@@ -690,7 +691,7 @@ scan_kernel(const __grid_constant__ ScanArgs a) {
   __shared__ double red[kReduceDoubles];
   __shared__ float dimc[3 * ZMC_MAX_N];
   const int64_t* fx = nullptr;
-  if constexpr (FxOf<F, PREC>::kTable != kFxNone) {
+  if constexpr (FxOf<F, PREC>::kTable == kFxCosTable || FxOf<F, PREC>::kTable == kFxExpTable) {
     __shared__ int64_t fx_table[FxOf<F, PREC>::kEntries];
     FxOf<F, PREC>::fill(fx_table);
     if (!a.stage_smem) __syncthreads();  // else stage_lists ends with one

@@ -130,6 +130,36 @@ def test_scale59(lib):
         assert abs((got if x < 5.65 else got % 2 ** 64) - want) <= 0.51
 
 
+@pytest.mark.parametrize("d", [1, 2, 5, 8])
+@pytest.mark.parametrize("x,a,b", [((0.5, 5.0), 0.0, 1.0), ((-3.0, 3.0), -1.0, 1.0),
+                                   ((1e6, 1e6), 0.0, 1.0), ((1.0, 2.0), 100.0, 101.0),
+                                   ((-5.0, -0.5), -2.0, 3.0), ((-1.001, -0.999), 0.9, 1.1)])
+def test_poly(lib, d, x, a, b):
+    """The root-mean-square error below 2^-52 of g's: a factor is rounded to 2^-60 of its
+    largest value and g once to FP64 (2^-54)."""
+    r = np.random.default_rng(d)
+    n = 400
+    xs = r.uniform(x[0], x[1], d)
+    v = r.integers(0, 2 ** 23, (n, d), dtype=np.uint32)
+    v[0], v[1] = 0, 2 ** 23 - 1
+    out = np.empty(n)
+    ptr = [z.ctypes.data_as(ctypes.c_void_p) for z in (xs, v, out)]
+    assert lib.fx_poly_n(ptr[0], f64(a), f64(b - a), ptr[1], ptr[2], ctypes.c_int(d),
+                         ctypes.c_int(n)) == 1
+    err, ref = [], []
+    for row, g in zip(v, out):
+        want = mpmath.mpf(1)
+        for xk, vk in zip(xs, row):
+            y = mpmath.mpf(a) + mpmath.mpf(b - a) * (2 * int(vk) + 1) / 2 ** 24
+            want *= 1 + mpmath.mpf(float(xk)) * y * y
+        err.append(float(mpmath.mpf(float(g)) - want))
+        ref.append(float(want))
+    assert np.sqrt(np.mean(np.square(err)) / np.mean(np.square(ref))) < 2.0 ** -52
+    bad = np.full(d, 1e30)
+    assert lib.fx_poly_n(bad.ctypes.data_as(ctypes.c_void_p), f64(a), f64(b - a), ptr[1], ptr[2],
+                         ctypes.c_int(d), ctypes.c_int(n)) == 0
+
+
 @pytest.mark.parametrize("n", [1, 2, 1000])
 def test_sum(lib, n):
     r = np.random.default_rng(n)

@@ -96,6 +96,30 @@ def test_gauss_ranges(zmc, N, lo, hi):
     assert np.all((np.abs(got["mean"] - ref["mean"]) <= tol) | nan)
 
 
+@pytest.mark.parametrize("N", [1, 2, 3, 5, 8])
+@pytest.mark.parametrize("lo,hi", [(0.0, 1.0), (-1.0, 1.0), (100.0, 101.5), (0.0, 1e-9),
+                                   (-1e20, 1e20)])
+def test_poly_ranges(zmc, N, lo, hi):
+    """Factors that change sign, cancel, are tiny, beyond 2^60 and not finite; the
+    oracle's rounding of 1 + x y^2 is 3 2^-53 of 1 + |x| y^2 per factor."""
+    x = np.array([0.0, 5e-324, -1e-300, 0.7, -0.3, -1.0, 5.0, 1e6, -1e9, 1e30, 1e100, np.inf,
+                  np.nan])
+    S, T = 1003, 2
+    a, b = np.full(N, lo), np.full(N, hi)
+    lists = [x] + [np.array([0.6])] * (N - 1)
+    with np.errstate(all="ignore"):
+        got, ref = _run(zmc, wl.G_POLY, N, a, b, lists, S, T)
+        V = (hi - lo) ** N
+        y2 = max(abs(lo), abs(hi)) ** 2
+        top = (1 + np.abs(x) * y2) * (1 + 0.6 * y2) ** (N - 1)
+        R = V * np.sqrt(np.mean(ref["s2"], axis=1) / S)
+        tol = 1e-12 * np.fmax(np.abs(ref["mean"]), R) + 4 * N * 2.0 ** -53 * V * top
+        same = np.isfinite(ref["mean"]) == np.isfinite(got["mean"])
+        ok = np.abs(got["mean"] - ref["mean"]) <= tol
+    assert np.all(same)
+    assert np.all(ok | ~np.isfinite(ref["mean"]))
+
+
 def test_unstaged_lists(zmc):
     """More list values than shared memory takes (read from global memory)."""
     r = np.random.default_rng(8)
