@@ -213,7 +213,7 @@ int batch_create(const zmc_scan_desc* d, zmc_scan_out* o, int n, int flags, zmc_
   cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
   // Philox calls per lane that give each precision's launch kBatchWaves lanes per
   // resident thread (two 256-thread blocks per SM), and trials per lane: as many
-  // as leave the launch kBatchRounds tiles per SM.
+  // as leave the launch batch_rounds tiles per SM.
   int64_t lane_calls[3] = {0, 0, 0};
   for (int i = 0; i < n; ++i) lane_calls[d[i].precision] += scan_calls(&d[i], counts[i]);
   for (auto& c : lane_calls) c /= kBatchWaves * 2 * kBatchBlock * std::max(sm, 1);
@@ -223,7 +223,7 @@ int batch_create(const zmc_scan_desc* d, zmc_scan_out* o, int n, int flags, zmc_
       plans[i] = plan_batch_scan(&d[i], b, lane_calls[d[i].precision], kBatchLeastGroups);
       tiles += batch_tiles(&d[i], counts[i], plans[i]);
     }
-    if (tiles >= kBatchRounds * std::max(sm, 1)) break;
+    if (tiles >= batch_rounds(b) * std::max(sm, 1)) break;
   }
 
   zmc_batch* b = new (std::nothrow) zmc_batch();

@@ -77,10 +77,12 @@ int64_t batch_tiles(const zmc_scan_desc* d, int64_t count, const TilePlan& tp);
 // 29 scans of 1.3e7 evaluations; 16 gives no more.
 constexpr int64_t kBatchWaves = 4;
 constexpr int64_t kBatchLeastGroups = 32;
-// Tiles per SM from which on lanes take several trials in the persistent kernel:
-// a launch with fewer is short of independent work (4.2e7 evaluations with four
-// trials per lane 1019 us, one 640 us; 5.4e9 in 6454 tiles 12.68 and 12.98 ms).
-constexpr int64_t kBatchRounds = 12;
+// Tiles per SM from which on lanes take b trials in the persistent kernel: a
+// launch with fewer is short of independent work, and its bodies spill registers
+// with four.  Measured: 4.2e7 evaluations with four trials per lane 1019 us, one
+// 640 us; 5.4e9 in 6500 tiles 12.98, 12.50, 12.67 ms with 1, 2, 4; 7.4e10 in
+// 10^5 tiles 226 and 224 ms with 2 and 4.
+constexpr int64_t batch_rounds(int b) { return b >= 4 ? 200 : b >= 2 ? 12 : 0; }
 // Lane groups of a launch over `count` points (and how many of them take four
 // and two trials, may be null).
 int64_t lane_groups_of(const zmc_scan_desc* d, int64_t count, const TilePlan& tp, int64_t* lu4,

@@ -717,7 +717,7 @@ int zmc_submit(zmc_server* s, const zmc_scan_desc* d, zmc_scan_out* o, uint64_t*
   const int64_t lane_calls = scan_calls(d, count) / (2 * kServeBlock * s->sm_count);
   for (int b = kMaxLaneTrials; b >= 1; b >>= 1) {
     r->tp = plan_batch_scan(d, b, lane_calls, kServeLeastGroups);
-    if (batch_tiles(d, count, r->tp) >= kBatchRounds * s->sm_count) break;
+    if (batch_tiles(d, count, r->tp) >= batch_rounds(b) * s->sm_count) break;
   }
   const int64_t per_point = int64_t(d->trials) * r->tp.splits;
   r->chunk_points = std::max<int64_t>(1, std::min<int64_t>(count, s->opts.chunk_units / per_point));
