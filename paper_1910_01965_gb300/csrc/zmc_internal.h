@@ -42,8 +42,12 @@ struct FieldConst {
   uint32_t shl4 = 16;            // shift left by 4
 };
 
-// Trials of one grid point that the same lanes sample together, at most.
+// Trials of one grid point that the same lanes sample together, at most: four, and
+// two from N = 6 on, where four spill registers.  Measured on GB300 against one
+// trial (FP32-Kahan, T = 8, 2e4 points, five integrands): two are 3-9 % faster at
+// every N; four 5-10 % at N = 1..5, but 2-5 %, 0-3 % and -2..3 % at N = 6, 7, 8.
 constexpr int kMaxLaneTrials = 4;
+constexpr int max_lane_trials(int N) { return N <= 5 ? kMaxLaneTrials : 2; }
 
 // Everything one launch of the sampling kernel needs, passed by value.
 // A "unit" is one (grid point, trial) pair; its S samples are cut into

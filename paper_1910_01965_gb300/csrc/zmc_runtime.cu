@@ -268,7 +268,8 @@ TilePlan plan_tiles(int N, int64_t S, int T, int64_t count, int sm_count,
 
 int max_lane_trials(const zmc_scan_desc* d) {
   if (d->precision == ZMC_FP64 || d->integrand_id == ZMC_G_CONST) return 1;
-  return d->trials >= 4 ? 4 : d->trials >= 2 ? 2 : 1;
+  const int most = max_lane_trials(d->N);
+  return d->trials >= 4 ? most : d->trials >= 2 ? 2 : 1;
 }
 
 // The launch shape.  Blocks of 128 threads: one warp per SM sub-partition, so that

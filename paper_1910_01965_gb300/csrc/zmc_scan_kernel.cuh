@@ -284,9 +284,9 @@ __device__ __forceinline__ auto eval_sample(const F& f, const FieldConst& fc,
 // A lane samples this many trials of one grid point together at most (they
 // share a part of every Philox call); the FP64 kernels, bound elsewhere, and the
 // constant integrand, which draws nothing, take one.
-template <class F, int PREC>
+template <int N, class F, int PREC>
 constexpr int max_trials() {
-  return PREC == kPrecFP64 || !F::kUsesSamples ? 1 : kMaxLaneTrials;
+  return PREC == kPrecFP64 || !F::kUsesSamples ? 1 : max_lane_trials(N);
 }
 
 // Sums over the sample groups [q, q_end) with stride `step` (one lane) of B
@@ -565,11 +565,13 @@ __device__ __forceinline__ void lane_sums(const ScanArgs& a, const uint32_t* rk0
     }
     if constexpr (FxOf<F, PREC>::kTable != kFxNoTable) f.fx = fx;
   }
-  if constexpr (max_trials<F, PREC>() > 1) {
+  if constexpr (max_trials<N, F, PREC>() > 2) {
     if (k.trials == 4) {
       sample_trials<N, F, PREC, 4>(a, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
       return;
     }
+  }
+  if constexpr (max_trials<N, F, PREC>() > 1) {
     if (k.trials == 2) {
       sample_trials<N, F, PREC, 2>(a, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
       return;
@@ -661,7 +663,7 @@ __device__ __forceinline__ void block_work(const ScanArgs& a, const uint32_t* rk
                                            const uint32_t* rk1, const void* table,
                                            const float* dimc, const int64_t* fx,
                                            int64_t first_w, int units, double* red) {
-  constexpr int kB = max_trials<F, PREC>();
+  constexpr int kB = max_trials<N, F, PREC>();
   const int lane = threadIdx.x & (a.lanes - 1);
   const int local = threadIdx.x >> a.lanes_log2;
   const bool active = local < units;
