@@ -6,8 +6,8 @@
 // block sums at once, all of one scan — and orders them longest first.  Each
 // resident block takes the next tile from a device counter (one atomicAdd by
 // thread 0, no waiting on other blocks), stages that scan's lists or constant
-// tables into shared memory when the scan changes, copies its Philox round
-// keys into registers, and runs the same per-lane sampling and reduction code
+// tables into shared memory when the scan changes, takes its Philox round
+// keys into uniform registers, and runs the same per-lane sampling and reduction code
 // as the single-scan kernel, writing each unit-split's FP64 partial sums into
 // that scan's slice of the batch's partial buffer.
 // The batched bodies keep as many Philox calls in flight per lane as the
@@ -50,13 +50,21 @@ __device__ __noinline__ void batch_tile(const ScanArgs& a, const BatchTile& t, b
   } else {
     table = a.stage_smem ? static_cast<const void*>(smem) : nullptr;
   }
+  // The round keys are the same for the whole warp: a reduction's result lives in
+  // uniform registers, which leaves 20 of the 128 to the body (spilled stores of the
+  // largest bodies 340-550 bytes without it, at most 200 with it; 64 uneven scans
+  // 12.50 -> 12.31 ms).
   uint32_t rk0[10], rk1[10];
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
-    rk0[r] = a.rk0[r];
-    rk1[r] = a.rk1[r];
+    rk0[r] = __reduce_or_sync(0xffffffffu, a.rk0[r]);
+    rk1[r] = __reduce_or_sync(0xffffffffu, a.rk1[r]);
   }
-  block_work<N, F, PREC>(a, rk0, rk1, table, dimc,
+  FieldConst fc;
+  fc.mask = __reduce_or_sync(0xffffffffu, a.field.mask);
+  fc.one = __reduce_or_sync(0xffffffffu, a.field.one);
+  fc.shl4 = __reduce_or_sync(0xffffffffu, a.field.shl4);
+  block_work<N, F, PREC>(a, fc, rk0, rk1, table, dimc,
                          FxOf<F, PREC>::kTable == kFxExpTable ? fxe : fxc, t.first_w, t.units,
                          red);
 }

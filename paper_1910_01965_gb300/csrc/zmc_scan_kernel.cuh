@@ -292,6 +292,14 @@ constexpr int max_trials() {
 // Sums over the sample groups [q, q_end) with stride `step` (one lane) of B
 // trials, trial u of them with the Philox constants b1[u], b2[u].
 //
+// What bounds the FP32 kernels: the ALU together with the FMA-heavy pipe.  On GB300
+// a LOP3 or shift holds the ALU for 2 clocks, and a 32x32->64 multiply the FMA-heavy
+// pipe for 4 and the ALU for 2 (probes: a multiply and n LOP3 take 2 + 2 n clocks,
+// a 32-bit multiply and a LOP3 together 2).  A call of B trials has 15 + 2/B such
+// multiplies, 17 + 2/B XORs and 8 field operations.  Gaussian N = 4, evaluations/s:
+// 4.49e11 at first, 4.69e11 with one ALU operation fewer per field, 4.84e11 with
+// B = 4 as well.
+//
 // Order of the compensated additions of a trial (the same for every blocking
 // choice below, so that the results do not depend on how many trials a lane
 // takes, and the single-scan and batched kernels agree bit for bit): with
@@ -442,10 +450,10 @@ __device__ __forceinline__ void lane_tail_group(const uint32_t* __restrict__ rk0
 // Sums of one lane over its part of split `split` of trials t .. t + B - 1 of
 // point p.
 template <int N, class F, int PREC, int B>
-__device__ __forceinline__ void sample_trials(const ScanArgs& a, const uint32_t* rk0,
-                                              const uint32_t* rk1, const F& f, int64_t p,
-                                              uint32_t t, int64_t split, int lane, double* s1,
-                                              double* s2) {
+__device__ __forceinline__ void sample_trials(const ScanArgs& a, const FieldConst& fc,
+                                              const uint32_t* rk0, const uint32_t* rk1,
+                                              const F& f, int64_t p, uint32_t t, int64_t split,
+                                              int lane, double* s1, double* s2) {
   constexpr int G = group_samples(N);
   typename FxOf<F, PREC>::Acc acc[B];
   const int64_t q0 = split * a.gps;
@@ -469,7 +477,7 @@ __device__ __forceinline__ void sample_trials(const ScanArgs& a, const uint32_t*
     const int64_t nfull = a.S / G;
     const int64_t qf = min(q1, nfull);
     if (q0 + lane < qf)
-      lane_groups<N, F, PREC, B>(rk0, rk1, pu[0].a2, pu[0].b0, b1, b2, f, a.field,
+      lane_groups<N, F, PREC, B>(rk0, rk1, pu[0].a2, pu[0].b0, b1, b2, f, fc,
                                  static_cast<uint32_t>(q0 + lane), static_cast<uint32_t>(qf),
                                  static_cast<uint32_t>(a.lanes), acc);
     if (G > 1) {
@@ -477,7 +485,7 @@ __device__ __forceinline__ void sample_trials(const ScanArgs& a, const uint32_t*
       if (valid > 0 && nfull >= q0 && nfull < q1 && ((nfull - q0) & (a.lanes - 1)) == lane)
 #pragma unroll
         for (int u = 0; u < B; ++u)
-          lane_tail_group<N, F>(rk0, rk1, pu[u], f, a.field, static_cast<uint32_t>(nfull), valid,
+          lane_tail_group<N, F>(rk0, rk1, pu[u], f, fc, static_cast<uint32_t>(nfull), valid,
                                 acc[u]);
     }
   }
@@ -497,7 +505,7 @@ __device__ __noinline__ void sample_unit_wide(const ScanArgs& a, const void* tab
                                               double* s2) {
   F f{};
   load_params<N>(a, table, static_cast<const float*>(nullptr), p, f);
-  sample_trials<N, F, PREC, 1>(a, a.rk0, a.rk1, f, p, t, split, lane, s1, s2);
+  sample_trials<N, F, PREC, 1>(a, a.field, a.rk0, a.rk1, f, p, t, split, lane, s1, s2);
 }
 
 // The work of the `lanes` threads of lane group w: `trials` trials from t on of
@@ -542,13 +550,14 @@ __device__ __forceinline__ LaneWork lane_work(const ScanArgs& a, int64_t w) {
 
 // Work of one lane of lane group w: decode, prepare, sample, sum; the sums of
 // its trials in s1, s2 (zero beyond them).  rk0/rk1 are the ten Philox round
-// keys (parameter space in the single-scan kernel, registers in the batched
-// one); fx the fixed-point functors' table.
+// keys (parameter space in the single-scan kernel, uniform registers in the
+// batched one); fx the fixed-point functors' table.
 template <int N, class F, int PREC>
-__device__ __forceinline__ void lane_sums(const ScanArgs& a, const uint32_t* rk0,
-                                          const uint32_t* rk1, const void* table,
-                                          const float* dimc, const int64_t* fx,
-                                          const LaneWork& k, int lane, double* s1, double* s2) {
+__device__ __forceinline__ void lane_sums(const ScanArgs& a, const FieldConst& fc,
+                                          const uint32_t* rk0, const uint32_t* rk1,
+                                          const void* table, const float* dimc,
+                                          const int64_t* fx, const LaneWork& k, int lane,
+                                          double* s1, double* s2) {
   const int64_t p = a.first + k.lp;
   if (!ZMC_CHECK(a.dbg, k.lp >= 0 && k.lp < a.count && k.split < a.splits &&
                             k.t + k.trials <= static_cast<uint32_t>(a.T),
@@ -567,17 +576,17 @@ __device__ __forceinline__ void lane_sums(const ScanArgs& a, const uint32_t* rk0
   }
   if constexpr (max_trials<N, F, PREC>() > 2) {
     if (k.trials == 4) {
-      sample_trials<N, F, PREC, 4>(a, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
+      sample_trials<N, F, PREC, 4>(a, fc, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
       return;
     }
   }
   if constexpr (max_trials<N, F, PREC>() > 1) {
     if (k.trials == 2) {
-      sample_trials<N, F, PREC, 2>(a, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
+      sample_trials<N, F, PREC, 2>(a, fc, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
       return;
     }
   }
-  sample_trials<N, F, PREC, 1>(a, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
+  sample_trials<N, F, PREC, 1>(a, fc, rk0, rk1, f, p, k.t, k.split, lane, s1, s2);
 }
 
 // Cross-warp sums of a block: 16 warps of up to 2 kMaxLaneTrials values.
@@ -659,10 +668,11 @@ __device__ __forceinline__ void write_sums(const ScanArgs& a, const LaneWork& k,
 // lanes): sample, reduce and write each trial's partial sums.  Every thread of
 // the block calls it.
 template <int N, class F, int PREC>
-__device__ __forceinline__ void block_work(const ScanArgs& a, const uint32_t* rk0,
-                                           const uint32_t* rk1, const void* table,
-                                           const float* dimc, const int64_t* fx,
-                                           int64_t first_w, int units, double* red) {
+__device__ __forceinline__ void block_work(const ScanArgs& a, const FieldConst& fc,
+                                           const uint32_t* rk0, const uint32_t* rk1,
+                                           const void* table, const float* dimc,
+                                           const int64_t* fx, int64_t first_w, int units,
+                                           double* red) {
   constexpr int kB = max_trials<N, F, PREC>();
   const int lane = threadIdx.x & (a.lanes - 1);
   const int local = threadIdx.x >> a.lanes_log2;
@@ -673,7 +683,7 @@ __device__ __forceinline__ void block_work(const ScanArgs& a, const uint32_t* rk
   for (int u = 0; u < 2 * kB; ++u) x[u] = 0.0;
   if (active) {
     k = lane_work<kB>(a, first_w + local);
-    lane_sums<N, F, PREC>(a, rk0, rk1, table, dimc, fx, k, lane, x, x + kB);
+    lane_sums<N, F, PREC>(a, fc, rk0, rk1, table, dimc, fx, k, lane, x, x + kB);
   }
   if constexpr (kB > 1) {
     // lane groups of one size lie together, the larger ones first
@@ -703,7 +713,7 @@ scan_kernel(const __grid_constant__ ScanArgs a) {
   const int per_block = blockDim.x >> a.lanes_log2;
   const int64_t first_w = static_cast<int64_t>(blockIdx.x) * per_block;
   const int64_t left = a.n_lw - first_w;
-  block_work<N, F, PREC>(a, a.rk0, a.rk1, table, dimc, fx, first_w,
+  block_work<N, F, PREC>(a, a.field, a.rk0, a.rk1, table, dimc, fx, first_w,
                          left < per_block ? static_cast<int>(left) : per_block, red);
 }
 
