@@ -16,31 +16,54 @@
 
 namespace zmc {
 
+// Trial t's sums over its splits, in order.
+__device__ __forceinline__ void trial_sums(const FinalizeArgs& a, const double* part, int t,
+                                           double* s1, double* s2) {
+  *s1 = *s2 = 0.0;
+  const double* pt = part + 2 * static_cast<int64_t>(t) * a.splits;
+  for (int k = 0; k < a.splits; ++k) {
+    *s1 += pt[2 * k];
+    *s2 += pt[2 * k + 1];
+  }
+}
+
+// Trials whose estimates are kept from the first pass to the second.
+constexpr int kKeptTrials = 8;
+
 // Point i's statistics from its 2 T splits partial sums at `part` (global or
-// shared memory), summed in a fixed order.
+// shared memory), summed in a fixed order.  The second pass over the trials needs
+// I_t again: up to kKeptTrials of them stay in registers, more are formed anew (the
+// same operations), for a division and the sums over the splits are what the kernel
+// spends its time on, on the SM's one FP64 unit.
 __device__ __forceinline__ void finalize_point_from(const FinalizeArgs& a, int64_t i,
                                                     const double* part) {
   const double S = static_cast<double>(a.S);
   double sumI = 0.0, pooled = 0.0;
-  for (int t = 0; t < a.T; ++t) {
-    double s1 = 0.0, s2 = 0.0;
-    const double* pt = part + 2 * static_cast<int64_t>(t) * a.splits;
-    for (int k = 0; k < a.splits; ++k) {
-      s1 += pt[2 * k];
-      s2 += pt[2 * k + 1];
-    }
+  double kept[kKeptTrials];
+  auto first_pass = [&](int t) {
+    double s1, s2;
+    trial_sums(a, part, t, &s1, &s2);
     if (a.s1) a.s1[i * a.T + t] = s1;
     if (a.s2) a.s2[i * a.T + t] = s2;
-    sumI += a.V * s1 / S;
-    pooled += (s2 - s1 * s1 / S) / (S - 1.0);
-  }
+    const double I = a.V * s1 / S;
+    sumI += I;
+    if (a.errw) pooled += (s2 - s1 * s1 / S) / (S - 1.0);
+    return I;
+  };
+#pragma unroll
+  for (int t = 0; t < kKeptTrials; ++t) kept[t] = t < a.T ? first_pass(t) : 0.0;
+  for (int t = kKeptTrials; t < a.T; ++t) first_pass(t);
   const double mean = sumI / a.T;
   double dev2 = 0.0;
   if (a.T > 1) {
-    for (int t = 0; t < a.T; ++t) {
-      const double* pt = part + 2 * static_cast<int64_t>(t) * a.splits;
-      double s1 = 0.0;
-      for (int k = 0; k < a.splits; ++k) s1 += pt[2 * k];
+#pragma unroll
+    for (int t = 0; t < kKeptTrials; ++t) {
+      const double dI = kept[t] - mean;
+      if (t < a.T) dev2 += dI * dI;
+    }
+    for (int t = kKeptTrials; t < a.T; ++t) {
+      double s1, s2;
+      trial_sums(a, part, t, &s1, &s2);
       const double dI = a.V * s1 / S - mean;
       dev2 += dI * dI;
     }
@@ -56,7 +79,7 @@ __device__ __forceinline__ void finalize_point(const FinalizeArgs& a, int64_t i)
 }
 
 // The partial sums of a block's points are one contiguous range.  When it fits
-// in shared memory (2 T splits <= 24 at 256 threads) the block first copies it
+// in shared memory (2 T splits <= 24 at 256 threads, 192 at 32) the block first copies it
 // with consecutive threads on consecutive doubles (coalesced reads), then each
 // thread sums its own point from shared memory; otherwise each thread reads its
 // point's sums from global memory.  The sums and their order are the same.
@@ -64,6 +87,7 @@ constexpr int kFinalizeStageDoubles = 6144;  // 48 KB
 
 __global__ void finalize_kernel(const __grid_constant__ FinalizeArgs a) {
   __shared__ double stage[kFinalizeStageDoubles];
+  cudaGridDependencySynchronize();  // the sampling kernel's sums (see finalize_launch)
   const int64_t first = static_cast<int64_t>(blockIdx.x) * blockDim.x;
   const int64_t n = min(static_cast<int64_t>(blockDim.x), a.count - first);
   const int64_t per = 2 * static_cast<int64_t>(a.T) * a.splits;
@@ -93,22 +117,37 @@ __global__ void finalize_batch_kernel(const __grid_constant__ FinalizeBatchArgs 
     finalize_point(b.fa[lo], k);
 }
 
+// Threads per block for n points: small, so that few points reach many SMs (a
+// point of five trials in six splits takes some 400 FP64 instructions, and an SM has
+// two FP64 lanes: 100 points in one block hold it for 9 us).  With the kept
+// estimates and the early launch below: the README call (100 points, five trials in
+// six splits) 88 -> 80 us, a call of 231 points 70 -> 66 us.
+static int finalize_block(int64_t n) { return n <= 32 * 152 ? 32 : n <= 128 * 152 ? 128 : 256; }
+
 int finalize_batch_launch(const FinalizeBatchArgs& a, void* stream) {
   if (a.total <= 0) return 0;
-  const int block = 256;
+  const int block = finalize_block(a.total);
   const int64_t grid = (a.total + block - 1) / block;
   finalize_batch_kernel<<<static_cast<unsigned>(grid), block, 0,
                           static_cast<cudaStream_t>(stream)>>>(a);
   return static_cast<int>(cudaGetLastError());
 }
 
+// Launched so that its blocks may start while the sampling kernel before it on the
+// stream ends; they wait for it (and its writes) before their first read.
 int finalize_launch(const FinalizeArgs& a, void* stream) {
   if (a.count <= 0) return 0;
-  const int block = 256;
-  const int64_t grid = (a.count + block - 1) / block;
-  finalize_kernel<<<static_cast<unsigned>(grid), block, 0,
-                    static_cast<cudaStream_t>(stream)>>>(a);
-  return static_cast<int>(cudaGetLastError());
+  const int block = finalize_block(a.count);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>((a.count + block - 1) / block));
+  cfg.blockDim = dim3(static_cast<unsigned>(block));
+  cfg.stream = static_cast<cudaStream_t>(stream);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return static_cast<int>(cudaLaunchKernelEx(&cfg, finalize_kernel, a));
 }
 
 // Raw words w = first_word + i of the stream of unit (p, t), through the same
