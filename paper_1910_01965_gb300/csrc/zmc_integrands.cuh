@@ -7,8 +7,9 @@
 // u = f - (1 - 2^-24) = (2 v + 1) 2^-24, y = a + (b - a) u.
 //
 // Two families:
-//  * FP64 functors (suffix 64, unit_t double) evaluate y and g in FP64, with
-//    the affine steps folded into per-unit constants as below.
+//  * FP64 functors (suffix 64Wide, unit_t double) evaluate y and g in FP64, with
+//    the affine steps folded into per-unit constants as below; those of the same
+//    integrands in fixed point are in zmc_integrands_fixed.cuh.
 //  * FP32 functors (suffix 32, unit_t float) take f as a float built from
 //    the field's bits, so y = (b - a) f + A with A = a - (b - a)(1 - 2^-24).
 //    Everything affine in y that depends only on (x, box) is folded, in
@@ -17,10 +18,13 @@
 //    cos/sin use the SFU (MUFU) approximations, exp uses ex2.approx.
 //
 // kCallsInFlight: independent Philox calls a lane keeps in flight per loop
-// block in the FP32 paths (measured on GB300: eight for the Gaussian,
-// cos-product and polynomial integrands, +1.6 % on the Gaussian at N = 4; four
-// for the others, whose N <= 3 kernels lose 1 % with eight).  The FP64 path
-// draws one group at a time (it is bound by its FP64 arithmetic).
+// block in the FP32 paths, over the trials it samples.  Measured on GB300, eight
+// against four: with one trial the cos-product, Gaussian, polynomial and
+// oscillatory kernels gain 0.5-3 % at N = 3 and 4 and change by -2.5..1 % at N = 1,
+// 2 and 5, with four trials they gain 1.4-3 % at N = 1 and nothing elsewhere; the
+// sine-sum loses 3 % at N = 4, so it and the user integrands keep four.  The FP64
+// path draws one group at a time (one sample's arithmetic has work enough to
+// overlap).
 // kFixedM > 0 marks a functor compiled for one number of parameters M (the
 // run-time-compiled user integrands); it receives parameter i by set_param.
 // `set(i, x_i, a_i, b_i)` receives parameter i and box side i (kPerDim: the
@@ -375,7 +379,7 @@ struct Osc32 {
   static constexpr bool kPerDim = true;
   static constexpr bool kTable = true;
   static constexpr bool kUsesSamples = true;
-  static constexpr int kCallsInFlight = 4;
+  static constexpr int kCallsInFlight = 8;
   static constexpr int kFixedM = 0;
   using unit_t = float;
   float W[N], A[N], X[N];

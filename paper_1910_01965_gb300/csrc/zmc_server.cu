@@ -712,6 +712,18 @@ int zmc_submit(zmc_server* s, const zmc_scan_desc* d, zmc_scan_out* o, uint64_t*
   r->user_out = o;
   r->o = *o;
   r->count = count;
+  const int64_t T = d->trials;
+  const auto size_request = [&]() {
+    const int64_t per_point = T * r->tp.splits;
+    r->chunk_points =
+        std::max<int64_t>(1, std::min<int64_t>(count, s->opts.chunk_units / per_point));
+    r->nchunks = count > 0 ? (count + r->chunk_points - 1) / r->chunk_points : 0;
+    r->out_doubles = static_cast<size_t>(r->chunk_points) * (3 + 2 * T);
+    const int nbuf = r->nchunks > 1 ? 2 : 1;
+    r->bytes = s256(nv * sizeof(double)) +
+               s256(static_cast<size_t>(r->chunk_points) * per_point * 16) +
+               nbuf * s256(r->out_doubles * sizeof(double));
+  };
   // Lanes short enough that the request alone gives every resident thread one
   // (it may be alone), and several trials per lane only if it keeps the GPU busy.
   const int64_t lane_calls = scan_calls(d, count) / (2 * kServeBlock * s->sm_count);
@@ -719,14 +731,11 @@ int zmc_submit(zmc_server* s, const zmc_scan_desc* d, zmc_scan_out* o, uint64_t*
     r->tp = plan_batch_scan(d, b, lane_calls, kServeLeastGroups);
     if (batch_tiles(d, count, r->tp) >= batch_rounds(b) * s->sm_count) break;
   }
-  const int64_t per_point = int64_t(d->trials) * r->tp.splits;
-  r->chunk_points = std::max<int64_t>(1, std::min<int64_t>(count, s->opts.chunk_units / per_point));
-  r->nchunks = count > 0 ? (count + r->chunk_points - 1) / r->chunk_points : 0;
-  const int64_t T = d->trials;
-  r->out_doubles = static_cast<size_t>(r->chunk_points) * (3 + 2 * T);
-  const int nbuf = r->nchunks > 1 ? 2 : 1;
-  r->bytes = s256(nv * sizeof(double)) + s256(static_cast<size_t>(r->chunk_points) * per_point * 16) +
-             nbuf * s256(r->out_doubles * sizeof(double));
+  size_request();
+  if (r->bytes > s->budget) {  // the longest lanes take the fewest partial sums
+    r->tp = plan_batch_scan(d, 1, INT64_MAX, kServeLeastGroups);
+    size_request();
+  }
   r->evals_total = static_cast<double>(count) * T * d->samples_per_point;
   r->evals_left = r->evals_total;
   r->t_submit = Clock::now();

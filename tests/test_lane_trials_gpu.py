@@ -77,3 +77,22 @@ def test_batches_of_all_sizes_equal_solo_runs(zmc, points, S, scans):
         assert np.array_equal(solo["s1"], res[2].cpu().numpy())
         assert np.array_equal(solo["s2"], res[3].cpu().numpy())
     zmc.zmc_batch_destroy(h)
+
+
+def test_server_budget_takes_the_longest_lanes(zmc):
+    """A request whose partial sums exceed the budget with short lanes (1 MB here, with
+    0.6 MB of lists and results) is planned with the longest ones and served."""
+    P, T, S = 2000, 8, 1 << 17
+    vals = np.linspace(0.5, 5.0, P)
+    args = (wl.G_COSPROD, 1, [0.0], [1.0], [P], vals, S, T, 3)
+    srv = zmc.Server(1 << 20)
+    try:
+        t = srv.submit(*args, want_sums=True)
+        assert srv.wait(t) == zmc.ZMC_OK
+        res, o = srv.result(t)
+        solo, _ = zmc.scan(*args, want_sums=True,
+                           tiles=(o.tile_lanes, o.tile_splits, o.tile_block))
+        assert np.array_equal(res["s1"], solo["s1"])
+        assert np.array_equal(res["mean"], solo["mean"])
+    finally:
+        srv.close()
