@@ -292,7 +292,7 @@ void plan_launch(const zmc_scan_desc* d, int64_t count, int sm, TilePlan* tp) {
   for (int i = 0; i < d->M; ++i) nvals += d->list_len[i];
   tp->launch_block = tp->block;
   // the caller's and the tuner's blocks stay as they are
-  if (d->tile_block == 0 && tp->block == 256 && tp->lanes <= 128 &&
+  if (d->tile_block == 0 && !tp->tuned && tp->block == 256 && tp->lanes <= 128 &&
       (nvals <= kLongLists || nvals > kMaxSmemVals))
     tp->launch_block = 128;
   const double per_block = static_cast<double>(tp->launch_block / tp->lanes);
@@ -395,6 +395,7 @@ static TilePlan plan_sums(const zmc_scan_desc* d, int64_t count, int sm, int tps
     }
     tp.lanes = tl;
     tp.block = tb;
+    tp.tuned = true;
     tp.splits = static_cast<int>(std::min<int64_t>(splits, std::max<int64_t>(1, Q)));
     return tp;
   }

@@ -17,6 +17,7 @@ struct TilePlan {
   // How the launch is shaped; neither changes a result.
   int trials = 1;          // trials of a point that the same lanes sample (1, 2, 4)
   int launch_block = 256;  // threads per block of the launch, at most `block`
+  bool tuned = false;      // lanes, splits and block are the autotuner's
 };
 
 // Byte offsets of each region inside one scan's device scratch.  The slice
@@ -78,10 +79,11 @@ int64_t batch_tiles(const zmc_scan_desc* d, int64_t count, const TilePlan& tp);
 constexpr int64_t kBatchWaves = 4;
 constexpr int64_t kBatchLeastGroups = 32;
 // Tiles per SM from which on lanes take b trials in the persistent kernel: a
-// launch with fewer is short of independent work, and its bodies spill registers
-// with four.  Measured: 4.2e7 evaluations with four trials per lane 1019 us, one
-// 640 us; 5.4e9 in 6500 tiles 12.98, 12.50, 12.67 ms with 1, 2, 4; 7.4e10 in
-// 10^5 tiles 226 and 224 ms with 2 and 4.
+// launch with fewer is short of independent work, and its largest bodies spill
+// registers with four.  Measured: 4.2e7 evaluations with four trials per lane
+// 1019 us, one 640 us; 5.4e9 in 6500 tiles 12.31 and 12.33 ms with 2 and 4 (12.98
+// with one, before the round keys took uniform registers); 7.4e10 in 10^5 tiles
+// 224.2 and 223.8 ms.
 constexpr int64_t batch_rounds(int b) { return b >= 4 ? 200 : b >= 2 ? 12 : 0; }
 // Lane groups of a launch over `count` points (and how many of them take four
 // and two trials, may be null).
