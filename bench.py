@@ -760,12 +760,15 @@ def run_registry(args):
                     meas["registers"] = m.get("registers")
                     meas["inst_per_eval"] = m.get("inst_per_eval")
                     line["measured_pipes"] = meas
-                    if p == zmc.ZMC_FP64 and m.get("fp64_sm_cycles_per_eval"):
+                    if p == zmc.ZMC_FP64 and "heavy" in meas and "fp64" in meas:
+                        # fixed point on the integer pipes, the sums on the FP64 unit
+                        bound = max(("heavy", "fp64"), key=lambda k: meas[k]["frac"])
                         line["roofline"] = {
-                            "bound": "fp64", "frac": meas["fp64"]["frac"],
-                            "basis": "FP64-pipe cycles per evaluation measured by ncu (the "
-                                     "FP64 cos/exp/sin are library routines; their operation "
-                                     "counts are not part of the method)"}
+                            "bound": "fma_heavy" if bound == "heavy" else "fp64",
+                            "frac": meas[bound]["frac"],
+                            "basis": "cycles per evaluation of the busiest pipe measured by "
+                                     "ncu (the operation counts of the 64-bit arithmetic are "
+                                     "not part of the method)"}
                 print(json.dumps(line), flush=True)
                 summary.append(line)
             del vals, mean, err

@@ -74,8 +74,8 @@ def _stamp() -> str:
 
 
 # The sources the single-scan sampling kernel is compiled from.
-KERNEL_SOURCES = ["zmc_scan_kernel.cuh", "zmc_integrands.cuh", "zmc_philox.cuh",
-                  "zmc_internal.h", "zmc_scan_inst.cu"]
+KERNEL_SOURCES = ["zmc_scan_kernel.cuh", "zmc_integrands.cuh", "zmc_integrands_fixed.cuh",
+                  "zmc_fixed64.cuh", "zmc_philox.cuh", "zmc_internal.h", "zmc_scan_inst.cu"]
 
 
 def source_stamp() -> str:

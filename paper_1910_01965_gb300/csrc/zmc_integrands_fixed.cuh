@@ -6,6 +6,18 @@
 // range; out of range, and for NaN or infinite parameters, the unit is sampled
 // by the FP64 functor named in FxOf (zmc_integrands.cuh, suffix Wide).
 //
+// What bounds them (ncu, registry grids): the FMA-heavy pipe, 82-87 % busy, and
+// beside it the ALU, which a multiply holds for 2 clocks too; the FP64 unit, 92 %
+// busy before, is left to the sums.  An N = 2 cosine product has 22 multiplies and
+// about 45 other operations per dimension.  GB300, evaluations/s before and after
+// (10^5-point grids): cos-product N = 1 2.6e10 -> 2.1e11, N = 8 3.4e9 -> 2.9e10;
+// Gaussian N = 4 2.3e10 -> 1.2e11; oscillatory N = 6 1.4e10 -> 7.9e10; polynomial
+// N = 1 1.1e11 -> 2.3e11, N = 8 1.7e10 -> 4.8e10.  Tables of 2048 steps, 20 and
+// 16 KB a block: the two 8-byte loads of a cosine take 12 shared-memory wavefronts
+// (31 % of the load unit); fewer steps need a further Taylor term, more shared
+// memory buys none less.  Products of 64-bit numbers with IMAD.WIDE and 64-bit
+// addends instead of high-half multiplies are 10 % slower.
+//
 // With u = (2 v + 1) 2^-24 and w = b - a (rounded to FP64, as there):
 // y = a + w 2^-24 + (w 2^-23) v.
 #pragma once
