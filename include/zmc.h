@@ -63,8 +63,8 @@ typedef enum {
  * width, or an integrand that cancels strongly, keeps only FP32's 24 bits;
  * ZMC_FP64 has no such limit.  Per sample the FP32 error is ~1e-7 of g. */
 typedef enum {
-  ZMC_FP64 = 0,        /* FP64 samples, integrand and sums (or 64-bit fixed
-                          point of at least that accuracy)                 */
+  ZMC_FP64 = 0,        /* FP64 samples, integrand and sums, or 64-bit fixed
+                          point where that is at least as accurate         */
   ZMC_FP32 = 1,        /* FP32 samples and integrand, plain FP32 lane sums  */
   ZMC_FP32_KAHAN = 2   /* FP32 samples and integrand, Kahan FP32 lane sums  */
 } zmc_precision;       /* cross-lane reduction and the statistics: FP64    */

@@ -3,10 +3,12 @@
 // GB300 has one FP64 unit per SM (2 lanes per clock: an FP64 instruction holds
 // it for 16 clocks a warp), against 32 lanes per clock for 32x32->64 integer
 // multiplies.  The FP64 integrands are therefore evaluated in 64-bit fixed
-// point on the integer pipes: every quantity carries at least as many
-// significant bits as an FP64 value of its size would, and the absolute error
-// of one evaluation is below 2^-56 (g is at most 1; one FP64 rounding of g is
-// 2^-54).  Two building blocks:
+// point on the integer pipes.  The cosine is held to an absolute 2^-56 (it is
+// at most 1; one FP64 rounding there is 2^-54), a product of cosines to 2^-60 and
+// g^2 to 2^-60 or 2^-62, so this holds what FP64 does only where g is not small all over the
+// box: the range tests (fx_mean_cos2, fx_cos_range) send the others to the FP64
+// functors.  The exponential and the polynomial keep their bits at any size.  Two
+// building blocks:
 //
 //  * phases in turns: theta = phase / (2 pi) mod 1 as a 64-bit fraction, so the
 //    reduction of the argument is integer wrap-around and costs nothing; cos of
@@ -48,6 +50,7 @@ ZMC_FX double fx_bits_double(uint64_t v) {
   return __longlong_as_double(static_cast<long long>(v));
 }
 ZMC_FX int fx_clz(uint32_t v) { return __clz(static_cast<int>(v)); }
+ZMC_FX float fx_cosf(float v) { return __cosf(v); }
 #else
 inline int32_t fx_mulhi(int32_t a, int32_t b) {
   return static_cast<int32_t>((static_cast<int64_t>(a) * b) >> 32);
@@ -69,6 +72,7 @@ inline double fx_bits_double(uint64_t u) {
   return v;
 }
 inline int fx_clz(uint32_t v) { return v ? __builtin_clz(v) : 32; }
+inline float fx_cosf(float v) { return __builtin_cosf(v); }
 #endif
 
 ZMC_FX int64_t fx_wide(int32_t a, int32_t b) { return static_cast<int64_t>(a) * b; }
@@ -149,6 +153,49 @@ ZMC_FX FxTurns fx_turns_mul(double a, double b, int k) {
 // |v| below 2^e (false for NaN and infinities); e within [-1000, 1000].
 ZMC_FX bool fx_below(double v, int e) {
   return static_cast<int>((fx_double_bits(v) >> 52) & 0x7ff) < 1023 + e;
+}
+
+// cos and sin of the turn with the leading 32 bits w, to about 2^-20.
+ZMC_FX float fx_cos_lead(uint32_t w) {
+  return fx_cosf(static_cast<float>(static_cast<int32_t>(w)) * 1.4629180792671596e-9f);
+}
+ZMC_FX float fx_sin_lead(uint32_t w) { return fx_cos_lead(w - 0x40000000u); }
+// The leading bits of 2^23 times a turn.
+ZMC_FX uint32_t fx_lead23(FxTurns t) { return (t.w2 << 23) | (t.w1 >> 9); }
+// sin(w) / w for w = `lead` in turns mod 1.
+ZMC_FX float fx_sinc(float w, uint32_t lead) {
+  return fabsf(w) < 0x1p-6f ? 1.0f - w * w * (1.0f / 6.0f) : fx_sin_lead(lead) / w;
+}
+// The mean of cos^2 over phases that are a sum of uniform ones: `centre2` is twice
+// the middle of their range in turns (leading bits), `sincs` the product of
+// sin(w) / w over the widths w.
+ZMC_FX float fx_mean_cos2(uint32_t centre2, float sincs) {
+  return 0.5f + 0.5f * fx_cos_lead(centre2) * sincs;
+}
+
+// Whether |cos| stays above 1/4 over the phases from `lead` (turns, leading bits)
+// to `width` radians further, or the phases reach over a radian.
+ZMC_FX bool fx_cos_range(uint32_t lead, float width) {
+  if (width >= 1.0f) return true;
+  const float a = fx_cos_lead(lead);
+  const float b = fx_cos_lead(lead + static_cast<uint32_t>(width * 683565275.6f));
+  return a * b > 0.0f && fabsf(a) >= 0.25f && fabsf(b) >= 0.25f;
+}
+
+// x y + q y^2 for y from a to a + w, q > 0: how far its values reach (`width`) and
+// by how much the lowest lies below the one at a (`drop`).
+struct FxReach {
+  float width, drop;
+};
+ZMC_FX FxReach fx_quad_reach(float x, float q, float a, float w) {
+  const float u = x + 2.0f * q * a;  // the slope at a
+  const float v = u + 2.0f * q * w;  // and at a + w
+  if (u < 0.0f && v > 0.0f) {        // lowest inside, at a - u / (2 q)
+    const float m = u * u / (4.0f * q), n = v * v / (4.0f * q);
+    return {m > n ? m : n, m};
+  }
+  const float d = w * (u + q * w);
+  return {fabsf(d), d < 0.0f ? -d : 0.0f};
 }
 
 // The 64-bit fraction of a turn plus half a table step: what fx_cos takes.
@@ -255,6 +302,19 @@ ZMC_FX int64_t fx_cos(uint64_t theta, const int64_t* table) {
 ZMC_FX int64_t fx_mul62(int64_t a, int64_t b) {
   const int64_t p = fx_mul(fx_top(a), fx_low(a), fx_top(b), fx_low(b), 1);
   return static_cast<int64_t>(static_cast<uint64_t>(p) << 2) + kFxBias;
+}
+
+// 2^SCALE g^2 for g = 2^62 g + 2^31, to about a unit (the cuts average out): 2^-60
+// with two multiplies of high halves, 2^-62 with the low half's whole product.
+template <int SCALE>
+ZMC_FX int64_t fx_square(int64_t g) {
+  static_assert(SCALE == 60 || SCALE == 62, "scale of the squares");
+  const int32_t h = fx_top(g), l = fx_low(g);
+  if constexpr (SCALE == 60) {
+    return fx_wide(h, h) + (2 * fx_mulhi(h, l) + 1);
+  } else {
+    return 4 * fx_wide(h, h) + ((fx_wide(h, l) + (1 << 28)) >> 29);
+  }
 }
 
 // -------------------------------------------------------------------- exp --

@@ -2,9 +2,19 @@
 //
 // Each functor evaluates its integrand from the sample's 23-bit fields with the
 // arithmetic of zmc_fixed64.cuh.  `set`/`finish` turn the box and the
-// parameters into fixed-point constants and decide (`ok`) whether they are in
-// range; out of range, and for NaN or infinite parameters, the unit is sampled
-// by the FP64 functor named in FxOf (zmc_integrands.cuh, suffix Wide).
+// parameters into fixed-point constants; `in_range` says whether they are large
+// and small enough for that.  Out of range, and for NaN or infinite parameters, the
+// unit is sampled by the FP64 functor named in FxOf (zmc_integrands.cuh, suffix
+// Wide).
+//
+// The cosines and sines have an absolute resolution (2^-56 in a cosine, 2^-60 in a
+// product and in g^2), so they are in range only where g is not small over the
+// whole box: R, the root mean square of g, follows from the phases' ranges.  The lines
+// lie where the error is no larger than the FP64 functor's, sample by sample, even in
+// boxes whose sides and parameters it represents without rounding.  Root mean square
+// over R and R^2 against 80-bit arithmetic, largest of some 800 boxes each, fixed point
+// over FP64: products g 0.91 (N = 1), 0.55 (2), 0.29 (8), g^2 0.91, 0.78, 0.77;
+// sine-sum g 1.00, g^2 0.96.  At R = 2^-6 instead g^2 is 5.6 times off for N = 2.
 //
 // What bounds them (ncu, registry grids): the FMA-heavy pipe, 82-87 % busy, and
 // beside it the ALU, which a multiply holds for 2 clocks too; the FP64 unit, 92 %
@@ -28,16 +38,15 @@
 namespace zmc {
 
 // Lane sums of values g with |g| <= 1, held as 2^62 g + 2^31: exact sums of g
-// and of g^2 to 2^-60 (rounded), converted to FP64 once per lane.  Integer sums
+// and of g^2 rounded to 2^-SCALE each, converted to FP64 once per lane.  Integer sums
 // cost 5 adds against 64 SMSP clocks for one FP64 add.
+template <int SCALE>
 struct FxLaneAcc {
   FxSum a1, a2;
   uint64_t n = 0;
   __device__ __forceinline__ void sum(int64_t g) {
     a1.add(g);
-    const int32_t h = fx_top(g);
-    const int32_t t = fx_mulhi(h, fx_low(g));
-    a2.add(fx_wide(h, h) + (2 * t + 1));
+    a2.add(fx_square<SCALE>(g));
   }
   __device__ __forceinline__ void add(int64_t g) {
     sum(g);
@@ -55,11 +64,12 @@ struct FxLaneAcc {
     n += K;
   }
   __device__ __forceinline__ double sum1() const { return a1.value(n, 62); }
-  __device__ __forceinline__ double sum2() const { return a2.value(0, 60); }
+  __device__ __forceinline__ double sum2() const { return a2.value(0, SCALE); }
 };
 
 // prod_k cos(x_k y_k): a 96-bit phase per dimension.  In range: phases below
-// 2^20 radians.
+// 2^20 radians; the mean of each factor's square over the box at least 2^-6, and of g^2
+// at least 2^-8 (N <= 5) or 2^-11 (the least over boxes that reach from 0 is 2^-10.8).
 template <int N>
 struct CosProd64 {
   static constexpr bool kPerDim = true;
@@ -70,6 +80,7 @@ struct CosProd64 {
   using unit_t = uint32_t;
   const int64_t* fx;
   bool ok = true;
+  float mean2 = 1.0f;  // of g^2
   uint32_t b0[N], b1[N], b2[N];
   uint64_t c[N];
   __device__ void set(int i, double xi, double ai, double bi) {
@@ -79,8 +90,14 @@ struct CosProd64 {
     b0[i] = b.w0;
     b1[i] = b.w1;
     b2[i] = b.w2;
-    c[i] = fx_phase0(fx_turns_add(fx_turns_mul(xi, ai, 0), fx_turns_sar(b, 1)));
+    const FxTurns xa = fx_turns_mul(xi, ai, 0);
+    c[i] = fx_phase0(fx_turns_add(xa, fx_turns_sar(b, 1)));
+    const uint32_t xw = fx_lead23(b);
+    const float m = fx_mean_cos2(2 * xa.w2 + xw, fx_sinc(static_cast<float>(xi * w), xw));
+    ok = ok && m >= 0x1p-6f;
+    mean2 *= m;
   }
+  __device__ bool in_range() const { return ok && mean2 >= (N <= 5 ? 0x1p-8f : 0x1p-11f); }
   __device__ int64_t eval(const uint32_t* v) const {
     int64_t g = fx_cos(fx_phase_step(c[0], v[0], b0[0], b1[0], b2[0]), fx);
 #pragma unroll
@@ -91,7 +108,8 @@ struct CosProd64 {
 };
 
 // sin(sum_k y_k + sum_l x_l) as the cosine a quarter turn behind.  In range:
-// the parameters' sum and the box's sides and corner below 2^20.
+// the parameters' sum and the box's sides and corner below 2^20; the mean of g^2 over
+// the box at least 2^-6.
 template <int N>
 struct SinSum64 {
   static constexpr bool kPerDim = false;
@@ -109,6 +127,8 @@ struct SinSum64 {
   __device__ void finish(const double* lo, const double* hi) {
     ok = fx_below(xsum, 20);
     FxTurns t = fx_turns_add(fx_turns(xsum, 0), {0, 0, 0xC0000000u});
+    uint32_t widths = 0;
+    float sincs = 1.0f;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
       const double w = hi[k] - lo[k];
@@ -118,9 +138,14 @@ struct SinSum64 {
       b1[k] = b.w1;
       b2[k] = b.w2;
       t = fx_turns_add(t, fx_turns_add(fx_turns(lo[k], 0), fx_turns_sar(b, 1)));
+      widths += fx_lead23(b);
+      sincs *= fx_sinc(static_cast<float>(w), fx_lead23(b));
     }
     c = fx_phase0(t);
+    // t lies half a field of each dimension (2^-24 of its width) above the corner
+    ok = ok && fx_mean_cos2(2 * t.w2 + widths, sincs) >= 0x1p-6f;
   }
+  __device__ bool in_range() const { return ok; }
   __device__ int64_t eval(const uint32_t* v) const {
     uint64_t th = c;
 #pragma unroll
@@ -138,7 +163,8 @@ __device__ __forceinline__ FxTurns fx_turns_quad(double a, double b, int k) {
 // cos(sum_k x_k y_k + 0.1 y_k^2).  In turns, dimension k adds
 //   (q v + l) v + const,  q = 0.1 w^2 2^-46,  l = (x w + 0.2 a w) 2^-23 + q,
 // by Horner's rule with q 2^23 and l held to 96 bits.  In range: box within
-// 2^10 of the origin, x w and x a below 2^20.
+// 2^10 of the origin, x w and x a below 2^20; phases that reach over a radian,
+// or over which |cos| stays above 1/4.
 template <int N>
 struct Osc64 {
   static constexpr bool kPerDim = true;
@@ -152,6 +178,7 @@ struct Osc64 {
   uint32_t q0[N], q1[N], q2[N];  // q 2^23, below 1/2
   uint32_t l0[N], l1[N], l2[N];
   uint64_t c = uint64_t(1) << 52;  // half a table step
+  float width = 0.0f, drop = 0.0f;  // of the phases' range
   __device__ void set(int i, double xi, double ai, double bi) {
     const double w = bi - ai;
     ok = ok && fx_below(xi * w, 20) && fx_below(xi * ai, 20) && fx_below(ai, 10) &&
@@ -172,6 +199,15 @@ struct Osc64 {
     const FxTurns k1 = fx_turns_add(fx_turns_sar(lin, 1), fx_turns_sar(q, 25));
     const FxTurns k = fx_turns_add(k0, k1);
     c += (static_cast<uint64_t>(k.w2) << 32) | k.w1;
+    const FxReach r = fx_quad_reach(static_cast<float>(xi), static_cast<float>(kOscQuad),
+                                    static_cast<float>(ai), static_cast<float>(w));
+    width += r.width;
+    drop += r.drop;
+  }
+  __device__ bool in_range() const {
+    const uint32_t at = static_cast<uint32_t>((c - (uint64_t(1) << 52)) >> 32);
+    return ok && (width >= 1.0f ||
+                  fx_cos_range(at - static_cast<uint32_t>(drop * 683565275.6f), width));
   }
   __device__ int64_t eval(const uint32_t* v) const {
     uint64_t th = c;
@@ -222,6 +258,7 @@ struct Gauss64 {
     c[i] = fx_scale59(s, kScale61) + fx_scale59(e, kScale61) +
            static_cast<int64_t>(((cw >> 23) + 1) >> 1) + kFxBias;
   }
+  __device__ bool in_range() const { return ok; }
   __device__ double eval(const uint32_t* v) const {
     uint64_t q = uint64_t(1) << 42;  // half a table step
 #pragma unroll
@@ -258,6 +295,7 @@ struct Poly64 {
     c1[i] = p.c1;
     c2[i] = p.c2;
   }
+  __device__ bool in_range() const { return ok; }
   __device__ double eval(const uint32_t* v) const {
     int64_t g = fx_poly_eval(c0[0], c1[0], c2[0], v[0]);
     int e = scale;
@@ -288,19 +326,20 @@ struct FxOf<Poly64<N>, kPrecFP64> {
   using Acc = LaneAcc<kPrecFP64>;
 };
 
-template <class W>
+template <class W, int SCALE = 60>
 struct FxCosOf {
   static constexpr int kTable = kFxCosTable;
   static constexpr int kEntries = kFxCosEntries;
   static constexpr size_t kStaticBytes = kEntries * sizeof(int64_t);
   using Wide = W;
-  using Acc = FxLaneAcc;
+  using Acc = FxLaneAcc<SCALE>;
   static __device__ __forceinline__ void fill(int64_t* dst) {
     fx_fill(dst, kFxTables.c, kEntries);
   }
 };
+// (products of four and more cosines are small enough to need the finer squares)
 template <int N>
-struct FxOf<CosProd64<N>, kPrecFP64> : FxCosOf<CosProd64Wide<N>> {};
+struct FxOf<CosProd64<N>, kPrecFP64> : FxCosOf<CosProd64Wide<N>, N <= 3 ? 60 : 62> {};
 template <int N>
 struct FxOf<SinSum64<N>, kPrecFP64> : FxCosOf<SinSum64Wide<N>> {};
 template <int N>

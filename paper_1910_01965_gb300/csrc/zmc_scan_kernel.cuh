@@ -567,7 +567,7 @@ __device__ __forceinline__ void lane_sums(const ScanArgs& a, const FieldConst& f
   F f{};
   load_params<N>(a, table, dimc, p, f);
   if constexpr (FxOf<F, PREC>::kTable != kFxNone) {
-    if (!f.ok) {
+    if (!f.in_range()) {
       sample_unit_wide<N, typename FxOf<F, PREC>::Wide, PREC>(a, table, p, k.t, k.split, lane,
                                                               s1, s2);
       return;

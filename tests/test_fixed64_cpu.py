@@ -168,3 +168,113 @@ def test_sum(lib, n):
         g = np.ascontiguousarray(g, np.int64)
         got = lib.fx_sum(g.ctypes.data_as(ctypes.c_void_p), ctypes.c_int(n), ctypes.c_int(62))
         assert got == float(mpmath.mpf(int(sum(int(v) for v in g))) / 2 ** 62)
+
+
+@pytest.mark.parametrize("scale", [60, 62])
+def test_square(lib, scale):
+    """g^2 to two units of 2^-scale, without a bias that grows with the sum."""
+    r = np.random.default_rng(6)
+    g = np.concatenate([r.integers(-2 ** 62, 2 ** 62, 4000), r.integers(-2 ** 50, 2 ** 50, 100),
+                        [2 ** 62, -2 ** 62, 0, 1, -1]])
+    got = _call(lib.fx_square_60 if scale == 60 else lib.fx_square_62, np.int64, len(g), g)
+    err = np.array([float(mpmath.mpf(int(q)) - mpmath.mpf(int(v)) ** 2 / 2 ** (124 - scale))
+                    for q, v in zip(got, g)])
+    assert np.max(np.abs(err)) <= 2.0
+    assert abs(err[:4000].mean()) < 5 * err[:4000].std() / np.sqrt(4000) + 0.4
+
+
+LD = np.longdouble
+
+
+def _cosprod(lib, d, x, a, w, v):
+    n = len(v)
+    m, least = np.zeros(1, np.float32), np.zeros(1, np.float32)
+    g, sq = np.empty(n, np.int64), np.empty(n, np.int64)
+    ptr = [z.ctypes.data_as(ctypes.c_void_p) for z in (x, v, m, least, g, sq)]
+    lib.fx_cosprod_n(ptr[0], f64(a), f64(w), ptr[1], d, n, *ptr[2:])
+    ok = least[0] >= 2.0 ** -6 and m[0] >= (2.0 ** -8 if d <= 5 else 2.0 ** -11)
+    return ok, float(m[0]), g, sq, 60 if d <= 3 else 62
+
+
+def _sinsum(lib, d, xsum, a, w, v):
+    n = len(v)
+    m, g, sq = np.zeros(1, np.float32), np.empty(n, np.int64), np.empty(n, np.int64)
+    ptr = [z.ctypes.data_as(ctypes.c_void_p) for z in (a, w, v, m, g, sq)]
+    lib.fx_sinsum_n(f64(xsum), *ptr[:3], d, n, *ptr[3:])
+    return m[0] >= 2.0 ** -6, float(m[0]), g, sq, 60
+
+
+def _judge(g, sq, scale, ex, n):
+    """Root-mean-square errors of g and of g^2 over R and R^2."""
+    R2 = np.mean(ex ** 2)
+    e1 = np.mean((g.astype(LD) * LD(2) ** -62 - ex) ** 2) / R2
+    e2 = np.mean((sq.astype(LD) * LD(2) ** -scale - ex ** 2) ** 2) / R2 ** 2
+    return float(np.sqrt(e1)), float(np.sqrt(e2)), float(R2)
+
+
+def test_range_of_small_cosines(lib):
+    """Boxes that the range tests let through, most of them near the line: the errors
+    of g below 2^-53 R and of g^2 below 2^-50 R^2 (one FP64 rounding is 2^-54.8 of a
+    value); the estimate of R^2 agrees with the samples' within their spread; and boxes
+    over which every factor is small, however many, are out."""
+    r = np.random.default_rng(7)
+    near = 0
+    for t in range(400):
+        d = int(r.integers(1, 9))
+        x = r.uniform(0.5, 5.0, d) if t % 4 == 0 else np.full(d, r.uniform(0.5, 5.0))
+        w = float(10 ** r.uniform(-2, 0.5))
+        a = float(r.uniform(-2, 2) if t % 4 == 0 else np.pi / 2 / x[0] - w * r.uniform())
+        v = r.integers(0, 2 ** 23, (500, d), dtype=np.uint32)
+        ok, m, g, sq, scale = _cosprod(lib, d, x, a, w, v)
+        y = LD(a) + LD(w) * (2 * v.astype(LD) + 1) * LD(2) ** -24
+        ex = np.cos(x.astype(LD) * y).prod(axis=1)
+        e1, e2, R2 = _judge(g, sq, scale, ex, len(v))
+        assert abs(m - R2) < 6 * float(np.std(ex ** 2)) / np.sqrt(500) + 1e-5, (d, x, a, w)
+        if ok:
+            near += m < 2.0 ** -6
+            assert e1 < 2.0 ** -53 and e2 < 2.0 ** -50, (d, x, a, w)
+    assert near > 20
+    for d, x, a, w in ((8, 3.0, 0.5, 0.05), (8, 1.0, 1.5, 0.1), (4, 1.0, 1.56, 0.02),
+                       (2, 3.14159, 0.499, 0.002), (6, 1.5, 1.0, 0.1), (8, 1.0, 1.0, 1.0)):
+        assert not _cosprod(lib, d, np.full(d, x), a, w, np.zeros((1, d), np.uint32))[0]
+
+
+def test_range_of_small_sines(lib):
+    r = np.random.default_rng(8)
+    for t in range(400):
+        d = int(r.integers(1, 9))
+        w, a = 10 ** r.uniform(-2, 0.3, d), r.uniform(-1, 1, d)
+        xsum = float(-a.sum() - w.sum() * r.uniform()) if t % 2 else float(r.integers(0, 400))
+        v = r.integers(0, 2 ** 23, (500, d), dtype=np.uint32)
+        ok, m, g, sq, scale = _sinsum(lib, d, xsum, a, w, v)
+        y = a.astype(LD) + w.astype(LD) * (2 * v.astype(LD) + 1) * LD(2) ** -24
+        ex = np.sin(y.sum(axis=1) + LD(xsum))
+        e1, e2, R2 = _judge(g, sq, scale, ex, len(v))
+        assert abs(m - R2) < 6 * float(np.std(ex ** 2)) / np.sqrt(500) + 1e-5
+        assert not ok or (e1 < 2.0 ** -53 and e2 < 2.0 ** -50)
+    for w in (1e-12, 1e-6, 0.2):
+        assert not _sinsum(lib, 1, 0.0, np.zeros(1), np.full(1, w), np.zeros((1, 1), np.uint32))[0]
+
+
+def test_range_of_oscillatory_phases(lib):
+    """The reach of x y + 0.1 y^2 against a fine grid, and |cos| over a stretch of
+    phases against its least there."""
+    r = np.random.default_rng(9)
+    out = np.empty(2, np.float32)
+    f32 = ctypes.c_float
+    for t in range(300):
+        x, a, w = r.uniform(-2, 2), r.uniform(-10, 10), 10 ** r.uniform(-2, 1)
+        if t % 2:
+            x = -0.2 * (a + w * r.uniform())  # lowest inside the box
+        lib.fx_quad(f32(x), f32(0.1), f32(a), f32(w), out.ctypes.data_as(ctypes.c_void_p))
+        y = a + w * np.linspace(0, 1, 20001)
+        p = x * y + 0.1 * y * y
+        size = abs(x) * w + 0.2 * (abs(a) + w) * w
+        assert abs(out[0] - np.ptp(p)) < 1e-5 * size and abs(out[1] - (p[0] - p.min())) < 1e-5 * size
+        start, width = r.uniform(0, 1), r.uniform(0, 1.2)
+        least = np.abs(np.cos(2 * np.pi * start + width * np.linspace(0, 1, 2001))).min()
+        got = lib.fx_range(u32(int(start * 2 ** 32)), f32(width))
+        if width >= 1.0:
+            assert got
+        elif abs(least - 0.25) > 1e-3:
+            assert bool(got) == (least > 0.25), (start, width)

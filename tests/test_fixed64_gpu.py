@@ -3,6 +3,7 @@ fixed-point integrands, in one grid, against the oracle."""
 import numpy as np
 import pytest
 
+import parity
 from oracle import oracle
 from paper_1910_01965_gb300 import workloads as wl
 
@@ -34,14 +35,34 @@ def _run(z, gid, N, lo, hi, lists, S, T=2, seed=3, tiles=(0, 0, 0)):
 
 def _compare(got, ref, N, lo, hi, S, phase):
     """1e-12 of scale, plus what FP64 keeps of the phase: the oracle rounds y and
-    each product, N 2^-52 of the largest |phase| (one row per grid point)."""
+    each product, N 2^-52 of the largest |phase| (one row per grid point).  An error
+    d of each g changes sum g^2 by at most 2 d sqrt(S sum g^2) + S d^2, the variance
+    that errw is formed from by what the two sums change, and errw by half of that
+    over errw, or by its root where errw is smaller."""
     V = float(np.prod(np.asarray(hi) - np.asarray(lo)))
+    T = ref["s1"].shape[1]
+    d = np.broadcast_to(N * 2.0 ** -52 * phase, ref["mean"].shape)[:, None]
+    rms = np.sqrt(ref["s2"] / S)
+    tol1 = 1e-12 * S * rms + S * d
+    with np.errstate(over="ignore"):
+        tol2 = 1e-12 * ref["s2"] + S * d * (2 * rms + d)
     R = V * np.sqrt(np.mean(ref["s2"], axis=1) / S)
-    tol = 1e-12 * np.maximum(np.abs(ref["mean"]), R) + V * N * 2.0 ** -52 * phase
-    ok = np.abs(got["mean"] - ref["mean"]) <= tol
-    nan = np.isnan(ref["mean"])
-    assert np.all(np.isnan(got["mean"]) == nan)
-    assert np.all(ok | nan), np.flatnonzero(~(ok | nan))
+    tols = {"s1": tol1, "s2": tol2,
+            "mean": 1e-12 * np.maximum(np.abs(ref["mean"]), R) + V * d[:, 0],
+            "err": 1e-12 * np.maximum(ref["err"], R) + 2 * V * d[:, 0]}
+    if S > 1:
+        dvar = np.mean(tol2 + 2 * np.abs(ref["s1"]) / S * tol1, axis=1) / (S - 1)
+        tols["errw"] = V * np.sqrt(dvar / (T * S))
+        with np.errstate(divide="ignore", invalid="ignore"):
+            half = V * V * dvar / (T * S) / (2 * ref["errw"])
+        tols["errw"] = 1e-12 * ref["errw"] + np.fmin(tols["errw"], half)
+    for name, tol in tols.items():
+        ok = np.abs(got[name] - ref[name]) <= tol
+        nan = np.isnan(ref[name])
+        if name != "errw":  # a negative variance of rounding errors is NaN in one only
+            assert np.all(np.isnan(got[name]) == nan), name
+        assert np.all(ok | nan | (name == "errw") & np.isnan(got[name])), \
+            (name, np.argwhere(~(ok | nan)))
 
 
 @pytest.mark.parametrize("S,tiles", [(1, (0, 0, 0)), (7, (0, 0, 0)), (1003, (0, 0, 0)),
@@ -128,3 +149,55 @@ def test_unstaged_lists(zmc):
     for gid, lo, hi in ((wl.G_COSPROD, 0.0, 1.0), (wl.G_GAUSS03, -1.0, 1.0)):
         got, ref = _run(zmc, gid, 1, [lo], [hi], [x], 41)
         _compare(got, ref, 1, [lo], [hi], 41, x * (gid == wl.G_COSPROD))
+
+
+# (integrand, N, parameter, box side) over which |g| is small everywhere: every
+# factor near a zero of the cosine, or the phase near a zero of the sine; and next
+# to them the bounds' edge, boxes where g is middling.
+SMALL_G = [(wl.G_COSPROD, 8, 3.0, 0.5, 0.55), (wl.G_COSPROD, 8, 1.0, 1.5, 1.6),
+           (wl.G_COSPROD, 4, 1.0, 1.56, 1.58), (wl.G_COSPROD, 2, 3.14159, 0.499, 0.501),
+           (wl.G_COSPROD, 8, 1.5, 1.0, 1.1), (wl.G_COSPROD, 6, 1.5, 1.0, 1.1),
+           (wl.G_COSPROD, 3, 1.0, 1.0, 2.0), (wl.G_COSPROD, 8, 1.0, 1.0, 2.0),
+           (wl.G_COSPROD, 1, 1.0, 1.5625, 1.578125), (wl.G_COSPROD, 8, 2.25, 0.0, 1.0),
+           (wl.G_SINSUM, 1, 0.0, 0.0, 1e-6), (wl.G_SINSUM, 2, 0.0, 0.0, 1e-9),
+           (wl.G_SINSUM, 1, 0.0, 0.0, 1e-12), (wl.G_SINSUM, 8, 0.0, -0.01, 0.01),
+           (wl.G_SINSUM, 1, 0.0, -0.125, 0.125), (wl.G_SINSUM, 3, 0.0, -1.0, 1.0),
+           (wl.G_OSC01, 1, 1.5, 0.979, 0.9835), (wl.G_OSC01, 2, 1.5, 0.506, 0.507),
+           (wl.G_OSC01, 1, 0.7927, -4.4, -3.53), (wl.G_OSC01, 3, 1.0, 0.3, 0.7)]
+
+
+@pytest.mark.parametrize("way", ["scan", "batch", "server"])
+@pytest.mark.parametrize("gid,N,x,lo,hi", SMALL_G)
+def test_small_integrands(zmc, gid, N, x, lo, hi, way):
+    """The sums and the statistics relative to their own size: 1e-12 of sum g^2 and of
+    the root mean square, whatever that is (parity.check), in grids that hold an
+    ordinary parameter beside the small one (where the box is wide enough for FP64 to
+    hold the spread of g that errw is formed from)."""
+    S, T = 2003, 3
+    lists = [np.array([x, x + (0.4 if hi - lo > 1e-3 else 0.0)])] + [np.array([x])] * (N - 1 if gid != wl.G_SINSUM else 0)
+    lens, vals = [len(v) for v in lists], np.concatenate(lists)
+    a, b = np.full(N, lo), np.full(N, hi)
+    args = (gid, N, a, b, lens, vals, S, T, 5)
+    ref = oracle.default().scan(*args, want_sums=True)
+    if way == "scan":
+        got, _ = zmc.scan(*args, precision=zmc.ZMC_FP64, want_sums=True)
+    elif way == "server":
+        srv = zmc.Server(1 << 28)
+        try:
+            t = srv.submit(*args, zmc.ZMC_FP64, want_sums=True)
+            assert srv.wait(t, 60000) == zmc.ZMC_OK
+            got, _ = srv.result(t)
+        finally:
+            srv.close()
+    else:
+        d, keep = zmc.make_desc(*args, zmc.ZMC_FP64)
+        got = {"mean": np.empty(2), "err": np.empty(2), "errw": np.empty(2),
+               "s1": np.empty((2, T)), "s2": np.empty((2, T))}
+        o = zmc.zmc_scan_out()
+        for k, v in got.items():
+            setattr(o, k, zmc._ptr(v))
+        zmc.zmc_scan_batch([d], [o])
+    V = float(np.prod(b - a))
+    parity.check(got, ref, V, S, 0, way)
+    assert np.all(np.abs(got["s2"] - ref["s2"]) <= 1e-12 * ref["s2"])
+    assert np.all(np.abs(got["s1"] - ref["s1"]) <= 1e-12 * np.sqrt(S * ref["s2"]))
