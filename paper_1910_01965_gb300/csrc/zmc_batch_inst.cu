@@ -123,30 +123,23 @@ batch_kernel(const __grid_constant__ BatchArgs b) {
 #define ZMC_BATCH_OCC2(p) batch_occupancy_p##p
 #define ZMC_BATCH_OCC(p) ZMC_BATCH_OCC2(p)
 
-// Shared memory above the default 48 KB has to be asked for; the FP64 kernel
-// holds both fixed-point tables beside the scans' lists.
-static cudaError_t allow_smem(size_t smem) {
+// The FP64 kernel holds both fixed-point tables beside the scans' lists.
 #if ZMC_INST_PREC == 0
-  const size_t fixed = (kFxCosEntries + kFxExpEntries) * sizeof(int64_t) + 1024;
+constexpr size_t kBatchTables = (kFxCosEntries + kFxExpEntries) * sizeof(int64_t);
 #else
-  const size_t fixed = 1024;
+constexpr size_t kBatchTables = 0;
 #endif
-  if (smem + fixed <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(batch_kernel<ZMC_INST_PREC>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(smem));
-}
 
 int ZMC_BATCH_FN(ZMC_INST_PREC)(const BatchArgs& b, int grid, int block, size_t smem,
                                 void* stream) {
-  const cudaError_t e = allow_smem(smem);
+  const cudaError_t e = allow_smem(batch_kernel<ZMC_INST_PREC>, kBatchTables, smem);
   if (e != cudaSuccess) return static_cast<int>(e);
   batch_kernel<ZMC_INST_PREC><<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(b);
   return static_cast<int>(cudaGetLastError());
 }
 
 int ZMC_BATCH_OCC(ZMC_INST_PREC)(int block, size_t smem, int* out) {
-  const cudaError_t e = allow_smem(smem);
+  const cudaError_t e = allow_smem(batch_kernel<ZMC_INST_PREC>, kBatchTables, smem);
   if (e != cudaSuccess) return static_cast<int>(e);
   return static_cast<int>(
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, batch_kernel<ZMC_INST_PREC>, block,

@@ -718,14 +718,25 @@ scan_kernel(const __grid_constant__ ScanArgs a) {
 }
 
 #ifndef __CUDACC_RTC__
+// Ask for more than the 48 KB of shared memory that a kernel gets unasked, where
+// `smem` bytes of lists beside `table_bytes` of tables may need it.  The limit belongs
+// to the kernel and not to the launch, so every call asks for the same, the longest
+// lists: no thread takes back what another is about to launch with.
+constexpr size_t kOtherSmem = 4096;  // bound of the sums', constants' and counters' arrays
+static_assert(kReduceDoubles * sizeof(double) + 3 * ZMC_MAX_N * sizeof(float) + 256 <= kOtherSmem,
+              "static shared memory beside the tables");
+template <class Kernel>
+cudaError_t allow_smem(Kernel kernel, size_t table_bytes, size_t smem) {
+  if (smem + table_bytes + kOtherSmem <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(kMaxSmemVals * sizeof(double)));
+}
+
 template <int N, class F, int PREC>
 int launch_scan(const ScanArgs& a, int block, int64_t grid, size_t smem, void* stream) {
-  if (smem + FxOf<F, PREC>::kStaticBytes + 1024 > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(scan_kernel<N, F, PREC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return static_cast<int>(e);
-  }
+  const cudaError_t e =
+      allow_smem(scan_kernel<N, F, PREC>, FxOf<F, PREC>::kStaticBytes, smem);
+  if (e != cudaSuccess) return static_cast<int>(e);
   scan_kernel<N, F, PREC><<<static_cast<unsigned>(grid), block, smem,
                             static_cast<cudaStream_t>(stream)>>>(a);
   return static_cast<int>(cudaGetLastError());
