@@ -267,7 +267,9 @@ TilePlan plan_tiles(int N, int64_t S, int T, int64_t count, int sm_count,
 }
 
 int max_lane_trials(const zmc_scan_desc* d) {
-  if (d->precision == ZMC_FP64 || d->integrand_id == ZMC_G_CONST) return 1;
+  if (d->precision == ZMC_FP64 || d->integrand_id == ZMC_G_CONST ||
+      is_user_integrand(d->integrand_id))
+    return 1;
   const int most = max_lane_trials(d->N);
   return d->trials >= 4 ? most : d->trials >= 2 ? 2 : 1;
 }
@@ -276,7 +278,10 @@ int max_lane_trials(const zmc_scan_desc* d) {
 // a short launch reaches all SMs and wastes less of its last turn; 256 where every
 // block stages a long list.  Measured on GB300 against 256-thread blocks: Gaussian
 // N = 4, T = 4, 2^14 samples, 10 points 53 -> 36 us, 700 points 144 -> 126 us;
-// with lists of 3000 values 464 -> 480 us.
+// with lists of 3000 values 464 -> 480 us.  User integrands keep 256 unless the launch
+// has fewer such blocks than SMs: one with a sine, two exponentials and a root per
+// dimension, 20,000 points, took 1184 (N = 1), 4458 (4) and 10,523 us (8) in blocks of
+// 256 and 1300, 4691 and 11,282 us in blocks of 128.
 //
 // Trials per lane: the number whose launch ends first by this model.  A block of
 // 4 (2) trials takes 3.7 (1.9) times as long as one of a single trial, having
@@ -291,14 +296,16 @@ void plan_launch(const zmc_scan_desc* d, int64_t count, int sm, TilePlan* tp) {
   int64_t nvals = 0;
   for (int i = 0; i < d->M; ++i) nvals += d->list_len[i];
   tp->launch_block = tp->block;
+  sm = std::max(1, sm);
+  const int64_t threads = count * d->trials * tp->splits * tp->lanes;  // of one trial each
   // the caller's and the tuner's blocks stay as they are
   if (d->tile_block == 0 && !tp->tuned && tp->block == 256 && tp->lanes <= 128 &&
-      (nvals <= kLongLists || nvals > kMaxSmemVals))
+      (nvals <= kLongLists || nvals > kMaxSmemVals) &&
+      (!is_user_integrand(d->integrand_id) || threads < int64_t(256) * sm))
     tp->launch_block = 128;
   const double per_block = static_cast<double>(tp->launch_block / tp->lanes);
   double best = 0.0;
   TilePlan t = *tp;
-  sm = std::max(1, sm);
   for (int b = 1; b <= max_lane_trials(d); b <<= 1) {
     t.trials = b;
     int64_t lu4 = 0, lu2 = 0;

@@ -1,0 +1,15 @@
+// C wrappers around the planner of csrc/zmc_runtime.h, linked with libzmc.so by
+// test_planner_cpu.py.
+#include "zmc_runtime.h"
+
+extern "C" int launch_shape(const zmc_scan_desc* d, int64_t count, int sm, int lanes, int splits,
+                            int block, int* out) {
+  zmc::TilePlan tp;
+  tp.lanes = lanes;
+  tp.splits = splits;
+  tp.block = block;
+  zmc::plan_launch(d, count, sm, &tp);
+  out[0] = tp.trials;
+  out[1] = tp.launch_block;
+  return 0;
+}
