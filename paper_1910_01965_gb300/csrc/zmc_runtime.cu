@@ -613,9 +613,16 @@ static void pinned_give(PinnedBuf b) {
 
 // Lists and outputs of a call that goes through a pinned buffer of this size.
 constexpr size_t kSmallCallBytes = size_t(1) << 18;
-// Blocks up to which they read the lists from host memory themselves (about a
-// microsecond each, against the copy's start-up on the stream).
+// The lists stay in the pinned buffer, read from there by up to so many blocks, where
+// every block stages few values or none.  Against a copy to the device first (cos-product,
+// N = 2, 50 to 6400 points): 0.5 to 1.5 us less with lists of 100 values, even at 300, 1 to
+// 3 us more at 1000 and 4 to 11 us more at 4000; 2 to 4 us less again above kMaxSmemVals,
+// where a block reads only the values of its points.
 constexpr int64_t kListReadBlocks = 2048;
+constexpr int64_t kListReadVals = 256;
+static bool read_lists_in_place(int64_t nvals, int64_t blocks) {
+  return blocks <= kListReadBlocks && (nvals <= kListReadVals || nvals > kMaxSmemVals);
+}
 
 // One output array of a chunk: where the finalize kernel wrote it on the
 // device, where it goes on the host, and its length in doubles.
@@ -694,7 +701,7 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
   const size_t per_chunk_doubles =
       static_cast<size_t>(cp) * (2 + (o->errw ? 1 : 0) + (o->s1 ? T : 0) + (o->s2 ? T : 0));
   // A small call with host buffers keeps the GPU's copy engine out: the lists go
-  // through a pinned buffer, from which the blocks read them if they are few, and
+  // through a pinned buffer, from which the blocks may read them themselves, and
   // the finalize kernel writes the results into it.  Two to three copies from and
   // into pageable memory took 18 us of the README call's 112 us.
   const size_t out_doubles = static_cast<size_t>(count) *
@@ -755,7 +762,7 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
   if (small) std::memcpy(stage.p, d->list_vals, nvals * sizeof(double));
   const int64_t blocks =
       lane_groups_of(d, count, tp, nullptr, nullptr) / (tp.launch_block / tp.lanes);
-  if (small && blocks <= kListReadBlocks) {
+  if (small && read_lists_in_place(nvals, blocks)) {
     vals_dev = reinterpret_cast<const double*>(stage.p);
   } else if (host) {
     double* v = reinterpret_cast<double*>(ws + L.vals);
