@@ -269,9 +269,9 @@ struct SinSum64Wide {
 // ------------------------------------------------------------------ FP32 --
 // FP32 functors with a per-value table (kTable): while the lists are staged
 // into shared memory each value x of list k becomes a float2 of per-value
-// constants (value(k, x, a, b)), and each dimension gets up to three FP32
-// per-dimension constants (dim(k, a, b, out)), both computed once per block in
-// FP64.  A thread then sets up a unit with table lookups only (load()).
+// constants (value(k, x, a, b); kValueChain: by several FP64 operations), and each
+// dimension gets up to three FP32 per-dimension constants (dim(k, a, b, out)), both
+// computed once per block in FP64.  A thread then sets up a unit with table lookups only (load()).
 
 template <int N>
 struct Const32 {
@@ -291,6 +291,7 @@ template <int N>
 struct CosProd32 {
   static constexpr bool kPerDim = true;
   static constexpr bool kTable = true;
+  static constexpr bool kValueChain = true;
   static constexpr bool kUsesSamples = true;
   static constexpr int kCallsInFlight = 8;
   static constexpr int kFixedM = 0;
@@ -317,6 +318,7 @@ template <int N>
 struct Gauss32 {
   static constexpr bool kPerDim = true;
   static constexpr bool kTable = true;
+  static constexpr bool kValueChain = true;
   static constexpr bool kUsesSamples = true;
   static constexpr int kCallsInFlight = 8;
   static constexpr int kFixedM = 0;
@@ -347,6 +349,7 @@ template <int N>
 struct Poly32 {
   static constexpr bool kPerDim = true;
   static constexpr bool kTable = true;
+  static constexpr bool kValueChain = false;
   static constexpr bool kUsesSamples = true;
   static constexpr int kCallsInFlight = 8;
   static constexpr int kFixedM = 0;
@@ -378,6 +381,7 @@ template <int N>
 struct Osc32 {
   static constexpr bool kPerDim = true;
   static constexpr bool kTable = true;
+  static constexpr bool kValueChain = false;
   static constexpr bool kUsesSamples = true;
   static constexpr int kCallsInFlight = 8;
   static constexpr int kFixedM = 0;
