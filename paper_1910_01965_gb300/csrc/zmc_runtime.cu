@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "zmc_internal.h"
+#include "zmc_pinned.h"
 #include "zmc_runtime.h"
 #include "zmc_trace.h"
 
@@ -569,47 +570,17 @@ static bool is_pinned_host(const void* p, size_t bytes) {
   return pinned(p) && pinned(static_cast<const char*>(p) + bytes - 1);
 }
 
-// Page-locked staging buffers for chunked scans into pageable host arrays and
-// for small calls, kept for reuse across calls (a process-wide free list; each
-// call holds its buffer for its duration, so concurrent calls never share one).
-struct PinnedBuf {
-  char* p = nullptr;
-  size_t bytes = 0;
+// Page-locked buffers: the results of chunked scans into pageable host arrays (the four
+// largest kept), and small calls, which have buffers of one size of their own, enough of
+// them for as many threads as call at once (up to 8 MiB kept).
+struct CudaHostMemory {
+  static int get(void** p, size_t bytes) {
+    return static_cast<int>(cudaHostAlloc(p, bytes, cudaHostAllocDefault));
+  }
+  static void put(void* p) { cudaFreeHost(p); }
 };
-static std::mutex g_pin_mu;
-static std::vector<PinnedBuf> g_pin_free;
-
-static int pinned_take(size_t bytes, PinnedBuf* out) {
-  {
-    std::lock_guard<std::mutex> lk(g_pin_mu);
-    for (size_t i = 0; i < g_pin_free.size(); ++i)
-      if (g_pin_free[i].bytes >= bytes) {
-        *out = g_pin_free[i];
-        g_pin_free.erase(g_pin_free.begin() + static_cast<long>(i));
-        return ZMC_OK;
-      }
-  }
-  PinnedBuf b;
-  cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&b.p), bytes, cudaHostAllocDefault);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaHostAlloc(staging)");
-  b.bytes = bytes;
-  *out = b;
-  return ZMC_OK;
-}
-
-static void pinned_give(PinnedBuf b) {
-  if (!b.p) return;
-  std::lock_guard<std::mutex> lk(g_pin_mu);
-  g_pin_free.push_back(b);
-  if (g_pin_free.size() > 4) {  // keep the four largest
-    auto it = std::min_element(g_pin_free.begin(), g_pin_free.end(),
-                               [](const PinnedBuf& x, const PinnedBuf& y) {
-                                 return x.bytes < y.bytes;
-                               });
-    cudaFreeHost(it->p);
-    g_pin_free.erase(it);
-  }
-}
+static PinnedPool<CudaHostMemory> g_chunk_buffers(4);
+static PinnedPool<CudaHostMemory> g_small_buffers(32);
 
 // Lists and outputs of a call that goes through a pinned buffer of this size.
 constexpr size_t kSmallCallBytes = size_t(1) << 18;
@@ -722,7 +693,7 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
       if (ready[b]) cudaEventDestroy(ready[b]);
       if (copied[b]) cudaEventDestroy(copied[b]);
     }
-    pinned_give(stage);
+    (small ? g_small_buffers : g_chunk_buffers).give(stage);
     if (own_ws) cudaFreeAsync(ws, stream);
   };
   if (piped) {
@@ -734,15 +705,19 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
         return cuda_fail(e, "cudaEventCreate");
       }
     }
-    if (!direct && (rc = pinned_take(2 * per_chunk_doubles * sizeof(double), &stage)) != ZMC_OK) {
+    const int e = direct ? 0 : g_chunk_buffers.take(2 * per_chunk_doubles * sizeof(double), &stage);
+    if (e != 0) {
       release();
-      return rc;
+      return cuda_fail(static_cast<cudaError_t>(e), "cudaHostAlloc(staging)");
     }
   }
 
-  if (small && (rc = pinned_take(kSmallCallBytes, &stage)) != ZMC_OK) {
-    release();
-    return rc;
+  if (small) {
+    const int e = g_small_buffers.take(kSmallCallBytes, &stage);
+    if (e != 0) {
+      release();
+      return cuda_fail(static_cast<cudaError_t>(e), "cudaHostAlloc(staging)");
+    }
   }
 
   // Events: 0 start, 1 lists copied, then per chunk (sampling start, sampling
