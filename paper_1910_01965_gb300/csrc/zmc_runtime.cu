@@ -680,8 +680,8 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
   int64_t list_doubles = 0;
   for (int i = 0; i < d->M; ++i) list_doubles += d->list_len[i];
   const size_t small_bytes = (static_cast<size_t>(list_doubles) + out_doubles) * sizeof(double);
-  const bool small = host && nch == 1 && !(d->flags & ZMC_F_TIMINGS) &&
-                     small_bytes <= kSmallCallBytes;
+  bool small = host && nch == 1 && !(d->flags & ZMC_F_TIMINGS) &&
+               small_bytes <= kSmallCallBytes;
   PinnedBuf stage;
   bool stage_in_use = false;  // by work enqueued on the stream
   cudaEvent_t ready[2] = {nullptr, nullptr}, copied[2] = {nullptr, nullptr};
@@ -712,12 +712,9 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
     }
   }
 
-  if (small) {
-    const int e = g_small_buffers.take(kSmallCallBytes, &stage);
-    if (e != 0) {
-      release();
-      return cuda_fail(static_cast<cudaError_t>(e), "cudaHostAlloc(staging)");
-    }
+  if (small && g_small_buffers.take(kSmallCallBytes, &stage) != 0) {
+    cudaGetLastError();
+    small = false;  // no page-locked memory to be had: by plain copies, as a larger call
   }
 
   // Events: 0 start, 1 lists copied, then per chunk (sampling start, sampling

@@ -1,10 +1,16 @@
 """Small calls with host buffers: lists and results go through a pinned buffer, which the
 kernels read and write themselves; the results are those of the same scan with device
 buffers, bit for bit, at either side of the sizes where the route changes."""
+import os
+import shutil
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -44,3 +50,38 @@ def test_host_equals_device(zmc, nvals, count, prec):
     torch.cuda.synchronize()
     for k in got:
         assert np.array_equal(got[k].ravel(), dev[k].cpu().numpy()), k
+
+
+# a cudaHostAlloc that always answers "out of memory" (2), in front of the real one
+NO_PINNED = "int cudaHostAlloc(void **p, unsigned long n, unsigned f) { return 2; }\n"
+CHILD = """
+import ctypes
+import numpy as np
+from paper_1910_01965_gb300 import zmc
+assert ctypes.CDLL(None).cudaHostAlloc(None, ctypes.c_ulong(8), 0) == 2
+v = np.linspace(0.5, 5, 20)
+mean, err = zmc.zmc_scan(1, 2, [0, 0], [1, 1], [10, 10], v, 1000, 3, 7)
+res, _ = zmc.scan(1, 2, [0, 0], [1, 1], [10, 10], v, 1000, 3, 7, want_sums=True)
+np.savez(%r, mean=mean, err=err, **{"r_" + k: a for k, a in res.items()})
+"""
+
+
+def test_without_page_locked_memory(zmc, tmp_path):
+    """Where no page-locked memory is to be had a small call still runs, by copies."""
+    gcc = shutil.which("gcc")
+    if not gcc:
+        pytest.skip("no gcc")
+    (tmp_path / "no.c").write_text(NO_PINNED)
+    so, out = str(tmp_path / "no.so"), str(tmp_path / "out.npz")
+    subprocess.run([gcc, "-shared", "-fPIC", "-o", so, str(tmp_path / "no.c")], check=True)
+    r = subprocess.run([sys.executable, "-c", CHILD % out], cwd=ROOT, capture_output=True,
+                       text=True, env=dict(os.environ, LD_PRELOAD=so), timeout=300)
+    assert r.returncode == 0, r.stderr[-1500:]
+    got = np.load(out)
+    v = np.linspace(0.5, 5, 20)
+    args = (1, 2, [0, 0], [1, 1], [10, 10], v, 1000, 3, 7)
+    mean, err = zmc.zmc_scan(*args)
+    res, _ = zmc.scan(*args, want_sums=True)
+    assert np.array_equal(got["mean"], mean) and np.array_equal(got["err"], err)
+    for k, a in res.items():
+        assert np.array_equal(got["r_" + k], a), k
