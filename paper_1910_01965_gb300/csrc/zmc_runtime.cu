@@ -298,11 +298,14 @@ void plan_launch(const zmc_scan_desc* d, int64_t count, int sm, TilePlan* tp) {
   for (int i = 0; i < d->M; ++i) nvals += d->list_len[i];
   tp->launch_block = tp->block;
   sm = std::max(1, sm);
-  const int64_t threads = count * d->trials * tp->splits * tp->lanes;  // of one trial each
-  // the caller's and the tuner's blocks stay as they are
+  // threads of one trial each
+  const double threads = static_cast<double>(count) * d->trials * tp->splits * tp->lanes;
+  // the caller's and the tuner's blocks stay as they are, and a grid that only the larger
+  // block brings below 2^31
   if (d->tile_block == 0 && !tp->tuned && tp->block == 256 && tp->lanes <= 128 &&
       (nvals <= kLongLists || nvals > kMaxSmemVals) &&
-      (!is_user_integrand(d->integrand_id) || threads < int64_t(256) * sm))
+      (!is_user_integrand(d->integrand_id) || threads < 256.0 * sm) &&
+      threads / 128 < 0x7fffffff)
     tp->launch_block = 128;
   const double per_block = static_cast<double>(tp->launch_block / tp->lanes);
   double best = 0.0;

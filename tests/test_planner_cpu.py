@@ -44,3 +44,12 @@ def test_user_integrands(plan):
         for count, block in ((1, 128), (10, 128), (606, 128), (608, 256), (40000, 256)):
             assert plan.shape(plan.zmc.ZMC_G_USER_BASE, N, 8, count, 8, 1) == (1, block)
     assert plan.shape(2, 4, 8, 40000, 4, 1)[0] > 1
+
+
+@pytest.mark.parametrize("lanes,points", [(128, 2 ** 31 - 2), (128, 2 ** 31 + 2), (32, 2 ** 33),
+                                          (128, 2 ** 32 - 4)])
+def test_grids_up_to_the_launch_limit(plan, lanes, points):
+    """What 256-thread blocks can launch stays launchable: no grid of 2^31 blocks."""
+    trials, block = plan.shape(2, 4, 1, points, lanes, 1, precision=0)
+    assert points // (block // lanes) <= 2 ** 31 - 1
+    assert block == (128 if points * lanes // 128 < 2 ** 31 - 1 else 256)
