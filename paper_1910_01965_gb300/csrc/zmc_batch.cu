@@ -106,6 +106,29 @@ int64_t batch_tiles(const zmc_scan_desc* d, int64_t count, const TilePlan& tp) {
   return (lane_groups_of(d, count, tp, nullptr, nullptr) + per_block - 1) / per_block;
 }
 
+// The plans of a batch's n scans of counts[i] points.  Each precision is a launch of its
+// own: lane_calls are the Philox calls per lane that give it kBatchWaves lanes per resident
+// thread (two 256-thread blocks per SM), and its lanes take as many trials as leave it
+// batch_rounds tiles per SM.
+void plan_batch(const zmc_scan_desc* d, const int64_t* counts, int n, int sm, TilePlan* plans) {
+  sm = std::max(sm, 1);
+  for (int prec = 0; prec < 3; ++prec) {
+    int64_t calls = 0;
+    for (int i = 0; i < n; ++i)
+      if (d[i].precision == prec) calls += scan_calls(&d[i], counts[i]);
+    const int64_t lane_calls = calls / (kBatchWaves * 2 * kBatchBlock * sm);
+    for (int b = kMaxLaneTrials; b >= 1; b >>= 1) {
+      int64_t tiles = 0;
+      for (int i = 0; i < n; ++i) {
+        if (d[i].precision != prec) continue;
+        plans[i] = plan_batch_scan(&d[i], b, lane_calls, kBatchLeastGroups);
+        tiles += batch_tiles(&d[i], counts[i], plans[i]);
+      }
+      if (tiles >= batch_rounds(b) * sm) break;
+    }
+  }
+}
+
 struct PrecGroup {
   int precision = -1;
   int64_t tile_begin = 0, tile_end = 0;
@@ -211,20 +234,7 @@ int batch_create(const zmc_scan_desc* d, zmc_scan_out* o, int n, int flags, zmc_
   int dev = 0, sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
-  // Philox calls per lane that give each precision's launch kBatchWaves lanes per
-  // resident thread (two 256-thread blocks per SM), and trials per lane: as many
-  // as leave the launch batch_rounds tiles per SM.
-  int64_t lane_calls[3] = {0, 0, 0};
-  for (int i = 0; i < n; ++i) lane_calls[d[i].precision] += scan_calls(&d[i], counts[i]);
-  for (auto& c : lane_calls) c /= kBatchWaves * 2 * kBatchBlock * std::max(sm, 1);
-  for (int b = kMaxLaneTrials; b >= 1; b >>= 1) {
-    int64_t tiles = 0;
-    for (int i = 0; i < n; ++i) {
-      plans[i] = plan_batch_scan(&d[i], b, lane_calls[d[i].precision], kBatchLeastGroups);
-      tiles += batch_tiles(&d[i], counts[i], plans[i]);
-    }
-    if (tiles >= batch_rounds(b) * std::max(sm, 1)) break;
-  }
+  plan_batch(d, counts.data(), n, sm, plans.data());
 
   zmc_batch* b = new (std::nothrow) zmc_batch();
   if (!b) return fail(ZMC_ENOMEM, "host allocation failed");

@@ -70,6 +70,8 @@ int64_t scan_calls(const zmc_scan_desc* d, int64_t count);
 TilePlan plan_batch_scan(const zmc_scan_desc* d, int trials, int64_t lane_calls,
                          int64_t least_groups);
 int64_t batch_tiles(const zmc_scan_desc* d, int64_t count, const TilePlan& tp);
+// The plans of the n scans of a batch on a device of `sm` SMs.
+void plan_batch(const zmc_scan_desc* d, const int64_t* counts, int n, int sm, TilePlan* plans);
 // A persistent launch gets this many lanes per resident thread, if they keep
 // kBatchLeastGroups sample groups each.  Measured on GB300 on small batches: 27
 // scans (4.2e7 evaluations) 640 us with lanes of up to 1024 groups whatever the

@@ -32,6 +32,20 @@ def plan(tmp_path_factory):
         lib.launch_shape(ctypes.byref(d), ctypes.c_int64(count), SM, lanes, splits, block, out)
         return out[0], out[1]
 
+    def batch(scans):
+        """(trials, lanes, splits) of each (integrand, N, points, samples, precision)."""
+        keep, descs = [], (zmc.zmc_scan_desc * len(scans))()
+        for i, (gid, N, points, S, precision) in enumerate(scans):
+            d, k = zmc.make_desc(gid, N, [0.0] * N, [1.0] * N, [points] + [1] * (N - 1), 0x1000,
+                                 S, 4, 0, precision, mem=zmc.ZMC_MEM_DEVICE)
+            keep.append(k)
+            descs[i] = d
+        counts = (ctypes.c_int64 * len(scans))(*[s[2] for s in scans])
+        out = (ctypes.c_int * (3 * len(scans)))()
+        lib.batch_trials(descs, counts, len(scans), SM, out)
+        return [tuple(out[3 * i:3 * i + 3]) for i in range(len(scans))]
+
+    lib.batch = batch
     lib.shape = launch_shape
     lib.zmc = zmc
     return lib
@@ -53,3 +67,14 @@ def test_grids_up_to_the_launch_limit(plan, lanes, points):
     trials, block = plan.shape(2, 4, 1, points, lanes, 1, precision=0)
     assert points // (block // lanes) <= 2 ** 31 - 1
     assert block == (128 if points * lanes // 128 < 2 ** 31 - 1 else 256)
+
+
+def test_batches_plan_each_precision_by_itself(plan):
+    """A precision's scans share a launch with none of the others, so their plans are
+    those of a batch of them alone."""
+    fp32 = [(2, 4, 64, 16384, 2)] * 10
+    fp64 = [(1, 2, 5000, 65536, 0)] * 40
+    plain = [(3, 3, 20000, 16384, 1)] * 5
+    alone = plan.batch(fp32) + plan.batch(fp64) + plan.batch(plain)
+    assert plan.batch(fp32 + fp64 + plain) == alone
+    assert alone[0][0] == 1 and alone[-1][0] > 1  # a short launch and a long one
