@@ -207,6 +207,13 @@ def load(path: str = LIBRARY):
         return lib
 
 
+def _points(lengths) -> int:
+    """Grid points of the lists' lengths (a sequence or one number); 0 where they overflow,
+    which the library then refuses."""
+    P = math.prod(np.asarray(lengths, np.int64).ravel().tolist())
+    return P if P <= 1 << 62 else 0
+
+
 def _addr(a: np.ndarray) -> int:
     return a.__array_interface__["data"][0]
 
@@ -267,7 +274,7 @@ def zmc_scan(gid, N, lo, hi, lengths, values, S, T, seed):
     hi = np.ascontiguousarray(hi, np.float64)
     L = np.ascontiguousarray(lengths, np.int64)
     v = np.ascontiguousarray(values, np.float64)
-    P = math.prod(L.tolist())
+    P = _points(L)
     mean = np.empty(P)
     err = np.empty(P)
     load()
@@ -534,7 +541,7 @@ def scan(gid, N, lo, hi, lengths, values, S, T, seed, precision=ZMC_FP32_KAHAN,
     d, keep = make_desc(gid, N, lo, hi, lengths, values, S, T, seed, precision,
                         ZMC_MEM_HOST, first_index, count, None, tiles, flags,
                         chunk_points=chunk_points)
-    P = math.prod(int(v) for v in lengths)
+    P = _points(lengths)
     n = (P - first_index) if count < 0 else count
     res = {"mean": np.empty(n), "err": np.empty(n)}
     if want_errw:

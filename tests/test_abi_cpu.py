@@ -115,6 +115,24 @@ def test_scan_without_gpu_fails_loudly(lib):
         lib.zmc_scan(1, 2, [0, 0], [1, 1], [10, 10], np.linspace(0.5, 5, 20), 64, 2, 0)
 
 
+def test_lengths_of_the_host_calls(lib):
+    """A product of lengths beyond 64 bits is the library's to refuse; one list's length
+    may be a number."""
+    vals = np.linspace(0.5, 5, 10)
+    for lens in ([2 ** 32, 2 ** 32], [2 ** 21] * 3, [2 ** 62, 2]):
+        N = len(lens)
+        for call in (lib.zmc_scan, lib.scan):
+            with pytest.raises(lib.ZmcError) as e:
+                call(1, N, [0] * N, [1] * N, lens, vals, 64, 2, 0)
+            assert e.value.status == lib.ZMC_EINVAL
+    for call in (lib.zmc_scan, lib.scan):
+        try:
+            res = call(1, 1, [0], [1], 10, vals, 64, 2, 0)
+            assert len(res[0]["mean"] if isinstance(res[0], dict) else res[0]) == 10
+        except lib.ZmcError:  # without a GPU
+            pass
+
+
 def test_integrand_registry(lib):
     names = [lib.zmc_integrand_info_get(i).name.decode() for i in range(lib.ZMC_G_COUNT)]
     assert names == ["const", "cosprod", "gauss03", "poly", "osc01", "sinsum"]
