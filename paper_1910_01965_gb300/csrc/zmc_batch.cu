@@ -157,6 +157,7 @@ struct zmc_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   int launches = 0;
+  int sm = 1;  // of the device
 };
 
 namespace zmc {
@@ -185,7 +186,7 @@ static int enqueue_run(zmc_batch* b, cudaStream_t s, cudaEvent_t mid) {
   fb.prefix = b->d_prefix;
   fb.nscans = b->n;
   fb.total = b->prefix[b->n];
-  const int fe = finalize_batch_launch(fb, s);
+  const int fe = finalize_batch_launch(fb, b->sm, s);
   if (fe != 0) return cuda_fail(static_cast<cudaError_t>(fe), "batched finalize launch");
   return ZMC_OK;
 }
@@ -239,6 +240,7 @@ int batch_create(const zmc_scan_desc* d, zmc_scan_out* o, int n, int flags, zmc_
   zmc_batch* b = new (std::nothrow) zmc_batch();
   if (!b) return fail(ZMC_ENOMEM, "host allocation failed");
   b->n = n;
+  b->sm = std::max(sm, 1);
   b->args.resize(n);
   b->fargs.resize(n);
   b->prefix.assign(n + 1, 0);

@@ -117,16 +117,18 @@ __global__ void finalize_batch_kernel(const __grid_constant__ FinalizeBatchArgs 
     finalize_point(b.fa[lo], k);
 }
 
-// Threads per block for n points: small, so that few points reach many SMs (a
+// Threads per block for n points on `sm` SMs: small, so that few points reach many SMs (a
 // point of five trials in six splits takes some 400 FP64 instructions, and an SM has
 // two FP64 lanes: 100 points in one block hold it for 9 us).  With the kept
 // estimates and the early launch below: the README call (100 points, five trials in
 // six splits) 88 -> 80 us, a call of 231 points 70 -> 66 us.
-static int finalize_block(int64_t n) { return n <= 32 * 152 ? 32 : n <= 128 * 152 ? 128 : 256; }
+static int finalize_block(int64_t n, int64_t sm) {
+  return n <= 32 * sm ? 32 : n <= 128 * sm ? 128 : 256;
+}
 
-int finalize_batch_launch(const FinalizeBatchArgs& a, void* stream) {
+int finalize_batch_launch(const FinalizeBatchArgs& a, int sm, void* stream) {
   if (a.total <= 0) return 0;
-  const int block = finalize_block(a.total);
+  const int block = finalize_block(a.total, sm);
   const int64_t grid = (a.total + block - 1) / block;
   finalize_batch_kernel<<<static_cast<unsigned>(grid), block, 0,
                           static_cast<cudaStream_t>(stream)>>>(a);
@@ -135,9 +137,9 @@ int finalize_batch_launch(const FinalizeBatchArgs& a, void* stream) {
 
 // Launched so that its blocks may start while the sampling kernel before it on the
 // stream ends; they wait for it (and its writes) before their first read.
-int finalize_launch(const FinalizeArgs& a, void* stream) {
+int finalize_launch(const FinalizeArgs& a, int sm, void* stream) {
   if (a.count <= 0) return 0;
-  const int block = finalize_block(a.count);
+  const int block = finalize_block(a.count, sm);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>((a.count + block - 1) / block));
   cfg.blockDim = dim3(static_cast<unsigned>(block));

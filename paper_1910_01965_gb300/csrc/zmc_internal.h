@@ -112,7 +112,7 @@ typedef int (*ScanLaunchFn)(const ScanArgs& a, int block, int64_t grid,
                             size_t smem, void* stream);
 
 ScanLaunchFn scan_launcher(int precision, int integrand, int N);
-int finalize_launch(const FinalizeArgs& a, void* stream);
+int finalize_launch(const FinalizeArgs& a, int sm, void* stream);
 
 // ------------------------------------------------------------- batches --
 // One tile = the lane groups one block sums at once, all of one scan.
@@ -143,7 +143,7 @@ int batch_launch(int precision, const BatchArgs& b, int grid, int block, size_t 
                  void* stream);
 // Blocks of the batched kernel that fit on one SM at `block` threads, `smem` bytes.
 int batch_blocks_per_sm(int precision, int block, size_t smem, int* out);
-int finalize_batch_launch(const FinalizeBatchArgs& a, void* stream);
+int finalize_batch_launch(const FinalizeBatchArgs& a, int sm, void* stream);
 
 int stream_words_launch(uint64_t seed, int64_t p, int t, uint64_t first_word,
                         int64_t nwords, uint32_t* out_dev, void* stream);

@@ -158,7 +158,7 @@ static int scan_noalloc(const zmc_scan_desc* d, zmc_scan_out* o) {
   f.s1 = o->s1;
   f.s2 = o->s2;
   f.dbg = a.dbg;
-  const int fe = finalize_launch(f, stream);
+  const int fe = finalize_launch(f, sm, stream);
   if (fe != 0) return cuda_fail(static_cast<cudaError_t>(fe), "finalize kernel launch");
   o->launches = 2;
   if (d->flags & ZMC_F_SYNC) {

@@ -843,7 +843,7 @@ int scan_ex(const zmc_scan_desc* d, zmc_scan_out* o) {
     f.errw = dev[2];
     f.s1 = dev[3];
     f.s2 = dev[4];
-    int e2 = finalize_launch(f, stream);
+    int e2 = finalize_launch(f, ds->prop.multiProcessorCount, stream);
     if (e2 != 0) {
       release();
       return cuda_fail(static_cast<cudaError_t>(e2), "finalize kernel launch");

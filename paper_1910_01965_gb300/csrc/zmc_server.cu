@@ -551,7 +551,7 @@ static void run_loop(zmc_server* s) {
         fb.prefix = reinterpret_cast<const int64_t*>(s->d_stage + off_pre);
         fb.nscans = static_cast<int32_t>(fa.size());
         fb.total = prefix.back();
-        if (finalize_batch_launch(fb, s->compute) != 0) rc = ZMC_ECUDA;
+        if (finalize_batch_launch(fb, s->sm_count, s->compute) != 0) rc = ZMC_ECUDA;
       }
       cudaEventRecord(s->ev_end[slot], s->compute);
       if (rc != ZMC_OK) {
