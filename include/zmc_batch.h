@@ -5,7 +5,11 @@
  * parameter grid (Sec. 2), exactly as zmc_scan_ex computes it: the same random
  * stream, the same per-unit sums, the same statistics, so a scan's results in
  * a batch are bit-identical to the same scan run alone with the same tile
- * configuration.  The paper runs batches of one grid on one GPU each (Sec. 2);
+ * configuration.  Where the descriptor leaves it open, the configuration
+ * depends on the device's SM count and on the total work of the batch's scans
+ * of the same precision (lanes are as short as that work needs to fill the
+ * GPU), so the last bits of a scan's sums do too; tile_lanes and tile_splits
+ * given in the descriptor pin them.  The paper runs batches of one grid on one GPU each (Sec. 2);
  * here scans of different integrands, dimensions, grid sizes and sample counts
  * share one launch: their work is cut into block-sized tiles, ordered longest
  * first, and taken by resident blocks from a device counter.

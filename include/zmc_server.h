@@ -5,7 +5,11 @@
  * of Eq. 1 over its parameter grid (Sec. 2), with the same random stream,
  * sums and statistics as zmc_scan_ex, so its results do not depend on what
  * else is being served (bit-identical to the same scan alone with the same
- * tile configuration; the configuration depends only on the request).
+ * tile configuration).  The configuration depends on the request and on the
+ * device's SM count; where its scratch would exceed the server's whole budget,
+ * on the budget too.  Lanes and splits fix the order of a unit's sums, so their
+ * last bits go with it; tile_lanes and tile_splits given in the descriptor pin
+ * them.
  *
  * A scheduler thread owns the GPU.  Requests wait in a queue and are admitted
  * at every step boundary while a slot is free and the device-memory budget

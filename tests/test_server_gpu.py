@@ -2,8 +2,9 @@
 cancellation, host-side failure injection, bounded waits.
 
 Every served result must equal the same scan run alone with the same tile
-configuration bit for bit: a request's tiles depend only on the request, and
-each tile computes the same sums whatever else shares the step.
+configuration bit for bit: a request's tiles depend on the request and the server
+(device, budget) and on nothing else that is being served, and each tile computes the
+same sums whatever else shares the step.
 """
 import threading
 import time
