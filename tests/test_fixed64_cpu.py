@@ -204,7 +204,7 @@ def _sinsum(lib, d, xsum, a, w, v):
     return m[0] >= 2.0 ** -6, float(m[0]), g, sq, 60
 
 
-def _judge(g, sq, scale, ex, n):
+def _errors(g, sq, scale, ex, n):
     """Root-mean-square errors of g and of g^2 over R and R^2."""
     R2 = np.mean(ex ** 2)
     e1 = np.mean((g.astype(LD) * LD(2) ** -62 - ex) ** 2) / R2
@@ -228,7 +228,7 @@ def test_range_of_small_cosines(lib):
         ok, m, g, sq, scale = _cosprod(lib, d, x, a, w, v)
         y = LD(a) + LD(w) * (2 * v.astype(LD) + 1) * LD(2) ** -24
         ex = np.cos(x.astype(LD) * y).prod(axis=1)
-        e1, e2, R2 = _judge(g, sq, scale, ex, len(v))
+        e1, e2, R2 = _errors(g, sq, scale, ex, len(v))
         assert abs(m - R2) < 6 * float(np.std(ex ** 2)) / np.sqrt(500) + 1e-5, (d, x, a, w)
         if ok:
             near += m < 2.0 ** -6
@@ -249,7 +249,7 @@ def test_range_of_small_sines(lib):
         ok, m, g, sq, scale = _sinsum(lib, d, xsum, a, w, v)
         y = a.astype(LD) + w.astype(LD) * (2 * v.astype(LD) + 1) * LD(2) ** -24
         ex = np.sin(y.sum(axis=1) + LD(xsum))
-        e1, e2, R2 = _judge(g, sq, scale, ex, len(v))
+        e1, e2, R2 = _errors(g, sq, scale, ex, len(v))
         assert abs(m - R2) < 6 * float(np.std(ex ** 2)) / np.sqrt(500) + 1e-5
         assert not ok or (e1 < 2.0 ** -53 and e2 < 2.0 ** -50)
     for w in (1e-12, 1e-6, 0.2):
